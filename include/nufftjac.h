@@ -167,6 +167,17 @@ int nufft_jvp_omega(nufft_plan_t p, int C, const nufft_cfloat* x, const nufft_cf
 int nufft_vjp_omega_x(nufft_plan_t p, int C, const nufft_cfloat* x, const nufft_cfloat* smaps,
                       const nufft_cfloat* v, float* grad_omega, nufft_cfloat* grad_x, void* stream);
 
+/* x = iters steps of conjugate gradients, from x = 0, on (E'E + lam I) x = b, the regularised
+ * normal equations of the CG-SENSE and PSD-inverse solves (Sec. II-F).  b and x are shaped as the
+ * adjoint's output ([N] with maps, [C][N] without, then one system over all images); they must not
+ * overlap.  `work` is nufft_cg_work_bytes bytes of device memory, 16-byte aligned, used until the
+ * work queued on `stream` has finished.  The whole solve is queued without waiting for the device:
+ * the scalars stay there, and the k-space values go from the gather to the spread in the sorted
+ * order, without passing through the caller's. */
+size_t nufft_cg_work_bytes(nufft_plan_t p, int C, int has_maps);
+int nufft_cg_normal(nufft_plan_t p, int C, const nufft_cfloat* b, const nufft_cfloat* smaps, float lam, int iters,
+                    nufft_cfloat* x, void* work, size_t work_bytes, void* stream);
+
 /* Device bytes a plan with these options, m points and calls of up to C coils would allocate
  * (C <= 0: o->max_coils).  Returns 0 for options nufft_plan would reject. */
 size_t nufft_workspace_bytes(const nufft_opts* o, int64_t m, int C);

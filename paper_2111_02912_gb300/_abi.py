@@ -26,7 +26,7 @@ EXPORTED = (
     "nufft_default_opts", "nufft_plan", "nufft_set_points", "nufft_sort_points", "nufft_forward", "nufft_adjoint",
     "nufft_jvp_omega", "nufft_vjp_omega_x", "nufft_workspace_bytes", "nufft_get_info", "nufft_destroy",
     "nufft_status_string", "nufft_last_error", "nufft_launch_count", "nufft_profile_enable",
-    "nufft_profile_read", "nufft_forward_noalloc",
+    "nufft_profile_read", "nufft_forward_noalloc", "nufft_cg_work_bytes", "nufft_cg_normal",
 )
 
 NUFFT_NOALLOC_SCRATCH_BYTES = 32 << 20
@@ -77,6 +77,10 @@ def lib():
         L.nufft_vjp_omega_x.argtypes = [vp, i32, vp, vp, vp, vp, vp, vp]
         L.nufft_forward_noalloc.argtypes = [ctypes.POINTER(nufft_opts), i64, vp, i32, vp, vp, vp, vp]
         L.nufft_forward_noalloc.restype = i32
+        L.nufft_cg_work_bytes.argtypes = [vp, i32, i32]
+        L.nufft_cg_work_bytes.restype = ctypes.c_size_t
+        L.nufft_cg_normal.argtypes = [vp, i32, vp, vp, ctypes.c_float, i32, vp, vp, ctypes.c_size_t, vp]
+        L.nufft_cg_normal.restype = i32
         L.nufft_workspace_bytes.argtypes = [ctypes.POINTER(nufft_opts), i64, i32]
         L.nufft_workspace_bytes.restype = ctypes.c_size_t
         L.nufft_get_info.argtypes = [vp, ctypes.POINTER(nufft_plan_info)]
@@ -144,6 +148,15 @@ def nufft_jvp_omega(plan, C, x, smaps, domega, dy, y_or_null, stream=0):
 
 def nufft_vjp_omega_x(plan, C, x, smaps, v, grad_omega, grad_x, stream=0):
     _check(lib().nufft_vjp_omega_x(plan, int(C), x, smaps, v, grad_omega, grad_x, stream), "nufft_vjp_omega_x")
+
+
+def nufft_cg_work_bytes(plan, C, has_maps):
+    return int(lib().nufft_cg_work_bytes(plan, int(C), int(bool(has_maps))))
+
+
+def nufft_cg_normal(plan, C, b, smaps, lam, iters, x, work, work_bytes, stream=0):
+    _check(lib().nufft_cg_normal(plan, int(C), b, smaps, float(lam), int(iters), x, work, int(work_bytes), stream),
+           "nufft_cg_normal")
 
 
 def nufft_workspace_bytes(opts, m, C=0):

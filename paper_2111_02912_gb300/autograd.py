@@ -135,12 +135,28 @@ def cg_solve(apply_F, b, iters, x0=None):
     return x
 
 
+def _solve_normal(op, b, lam, iters):
+    """iters CG steps on (E'E + lam I) x = b: the library's solver where it applies, else cg_solve.
+
+    The solver takes the operator as it is (its own E and E', not a subclass's or a replaced method)
+    and b shaped like the adjoint's output.  One step of the vector algebra is three launches there
+    and about twenty small ones here, which held the GPU up: psd_inverse and its gradient at 320^2,
+    16 coils, 51,200 points, ten iterations each way: 6732 -> 2957 us.
+    """
+    one = op.smaps is not None if isinstance(op, NufftOperator) else False
+    plain = (type(op) is NufftOperator and type(op.plan) is Plan and b.is_cuda and b.dtype == torch.complex64
+             and not {"forward", "adjoint"} & op.__dict__.keys() and isinstance(lam, (int, float)) and iters > 0
+             and tuple(b.shape if one else b.shape[1:]) == op.shape)
+    if plain:
+        return op.plan.cg_normal(b.resolve_conj().contiguous(), lam, iters, op.smaps)
+    return cg_solve(lambda v: op.adjoint(op.forward(v)) + lam * v, b, iters)
+
+
 class _PsdInverse(torch.autograd.Function):
     @staticmethod
     def forward(ctx, b, omega, op, lam, iters):
         op.sync(omega)
-        F = lambda v: op.adjoint(op.forward(v)) + lam * v
-        z = cg_solve(F, b.contiguous(), iters)
+        z = _solve_normal(op, b.contiguous(), lam, iters)
         ctx.op, ctx.lam, ctx.iters = op, lam, iters
         ctx.save_for_backward(z, omega)
         return z
@@ -150,8 +166,7 @@ class _PsdInverse(torch.autograd.Function):
         z, omega = ctx.saved_tensors
         op, lam = ctx.op, ctx.lam
         op.sync(omega)
-        F = lambda v: op.adjoint(op.forward(v)) + lam * v
-        u = cg_solve(F, g.contiguous(), ctx.iters)                 # u = F^-1 g
+        u = _solve_normal(op, g.contiguous(), lam, ctx.iters)      # u = F^-1 g
         go = None
         if ctx.needs_input_grad[1]:                                 # Eq. (e,inv,omd)
             go = -(op.vjp_omega(z, op.forward(u)) + op.vjp_omega(u, op.forward(z)))

@@ -309,6 +309,7 @@ struct GatherArgs {
     float* grad;          // [D][M]
     float2* v_sorted;     // VJP: if set, v is also written here in sorted point order, [C][M]
     int v_sorted_cpt;     // ... in the strip layout [C / cpt][M][cpt] instead, when > 0
+                          // (forward: with both set, y goes there in the strip layout, not to y)
 };
 // cpl: lane slots per lane (coils l + k G), or 0 for coil pairs, kGatherQuads for coil quads
 constexpr int kGatherQuads = -4;
@@ -362,6 +363,17 @@ cudaError_t launch_spread(const SpreadArgs& a, int cpl, cudaStream_t s, size_t s
 cudaError_t launch_zero_heavy_tiles(const SpreadArgs& a, cudaStream_t s);
 // ys[c][i] = y[c][idx[i].w]: the coil values in sorted point order (coalesced reads in the spread).
 cudaError_t launch_permute_y(const int4* idx, const float2* y, float2* ys, int64_t M, int C, cudaStream_t s);
+// Vector steps of CG on (E'E + lam I) x = b (kernels_cg.cu); per-block partial sums in pq, rr, rr_new.
+constexpr int kCgBlocks = 608;   // four 256-thread blocks per SM
+enum CgStep { CG_START, CG_DOT, CG_UPDATE, CG_DIR };
+struct CgArgs {
+    int64_t n;
+    float lam;
+    const float2* b;
+    float2 *x, *r, *p, *q;             // [n]; q = E'E p
+    double *pq, *rr, *rr_new;          // [kCgBlocks]
+};
+cudaError_t launch_cg(CgStep step, const CgArgs& a, cudaStream_t s);
 int spread_min_slots(int D, int J);   // fewest tap slots per warp the spread kernel supports
 // Tile spread (row owners in 2-D, cell owners in 3-D): D in {2, 3}, every tile edge <= K - J + 1 and >= J - 1, prod B <= 512,
 // a.CC = coils per block (4, 8 or 16), a.P candidates per work item (<= prod B).

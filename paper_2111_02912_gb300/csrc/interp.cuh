@@ -157,8 +157,16 @@ __device__ __forceinline__ void gather_body(const GatherArgs& a) {
 #pragma unroll
         for (int k = 0; k < CPL; ++k)
 #pragma unroll
-            for (int i = 0; i < W; ++i)
-                if (ok[k]) a.y[(int64_t)(W * (lane_g + k * G) + i) * M + orig] = acc[0][k][i];
+            for (int i = 0; i < W; ++i) {
+                if (!ok[k]) continue;
+                const int c = W * (lane_g + k * G) + i;
+                if (a.v_sorted_cpt) {   // for the adjoint spread of the same points
+                    const int cg = c / a.v_sorted_cpt;
+                    a.v_sorted[((int64_t)cg * M + pt) * a.v_sorted_cpt + (c - cg * a.v_sorted_cpt)] = acc[0][k][i];
+                } else {
+                    a.y[(int64_t)c * M + orig] = acc[0][k][i];
+                }
+            }
     } else if (MODE == GM_JVP) {
         float dom[D];
 #pragma unroll

@@ -37,13 +37,13 @@ int fail(int status, const std::string& msg) {
 enum ProfKind {
     PK_ZERO, PK_BIN_COUNT, PK_BIN_SCAN, PK_TILE_SCAN, PK_BIN_SCATTER, PK_BIN_ITEMS, PK_FFT_FWD_FIRST, PK_FFT_FWD_MID,
     PK_FFT_INV_MID, PK_FFT_INV_LAST, PK_GATHER_FWD, PK_GATHER_JVP, PK_GATHER_VJP, PK_ZERO_HEAVY, PK_SPREAD, PK_SUM_CHUNKS, PK_PERMUTE_Y,
-    PK_STRIP_PLAN_A, PK_STRIP_PLAN_B, PK_STRIP_FILL, PK_DET_PLACE, PK_DET_RANK, PK_STRIP_ORDER, PK_COUNT
+    PK_STRIP_PLAN_A, PK_STRIP_PLAN_B, PK_STRIP_FILL, PK_DET_PLACE, PK_DET_RANK, PK_STRIP_ORDER, PK_CG, PK_COUNT
 };
 const char* kProfNames[PK_COUNT] = {"zero", "bin_count", "bin_scan", "tile_scan", "bin_scatter", "bin_items", "fft_fwd_first",
                                     "fft_fwd_mid", "fft_inv_mid", "fft_inv_last", "gather_fwd", "gather_jvp",
                                     "gather_vjp", "zero_heavy", "spread", "sum_chunks", "permute_y",
                                     "strip_plan_a", "strip_plan_b", "strip_fill", "det_place", "det_rank",
-                                    "strip_order"};
+                                    "strip_order", "cg"};
 
 int64_t grid_size(int64_t n, double sigma) {
     int64_t k = (int64_t)std::ceil(sigma * (double)n - 1e-9);
@@ -1259,6 +1259,61 @@ int nufft_vjp_omega_x(nufft_plan_t p, int C, const nufft_cfloat* x, const nufft_
     if ((st = sort_join(p, s))) return st;
     if (grad_x) st = adjoint_impl(p, C, (const float2*)v, (const float2*)smaps, (float2*)grad_x, s, vsorted);
     return finish_call(p, s, st);
+}
+
+// Vectors r, p and q, the k-space values of a plan without strips, and the partial sums.
+size_t nufft_cg_work_bytes(nufft_plan_t p, int C, int has_maps) {
+    if (!p || C < 1 || C > p->maxC) return 0;
+    const size_t n = (size_t)p->Nimg * (has_maps ? 1 : C);
+    return (3 * n + (p->strip ? 0 : (size_t)C * p->M)) * sizeof(float2) + 3 * kCgBlocks * sizeof(double);
+}
+
+int nufft_cg_normal(nufft_plan_t p, int C, const nufft_cfloat* b, const nufft_cfloat* smaps, float lam, int iters,
+                    nufft_cfloat* x, void* work, size_t work_bytes, void* stream) {
+    int st;
+    if ((st = check_call(p, C))) return st;
+    if (!b || !x || !work || iters < 0) return fail(NUFFT_ERR_INVALID_ARG, "b, x or work is NULL, or iters < 0");
+    if (work_bytes < nufft_cg_work_bytes(p, C, smaps != nullptr))
+        return fail(NUFFT_ERR_INVALID_ARG, "work is smaller than nufft_cg_work_bytes");
+    cudaStream_t s = (cudaStream_t)stream;
+    p->last_stream = s;
+    if ((st = sort_rest(p, s))) return st;
+    CgArgs a{};
+    a.n = p->Nimg * (smaps ? 1 : C);
+    a.lam = lam;
+    a.b = (const float2*)b;
+    a.x = (float2*)x;
+    a.pq = (double*)work;
+    a.rr = a.pq + kCgBlocks;
+    a.rr_new = a.rr + kCgBlocks;
+    a.r = (float2*)(a.rr_new + kCgBlocks);
+    a.p = a.r + a.n;
+    a.q = a.p + a.n;
+    float2* y = a.q + a.n;   // plans without strips only
+    const int cpt = 64 / p->NSL;
+    auto cg = [&](CgStep step) { return launch(p, PK_CG, s, [&] { return launch_cg(step, a, s); }); };
+    if ((st = cg(CG_START))) return st;
+    for (int k = 0; k < iters; ++k) {
+        if (p->M > 0) {
+            if ((st = forward_grids(p, C, 1, 1, a.p, (const float2*)smaps, s))) return st;
+            if ((st = sort_join(p, s))) return st;
+            GatherArgs g = gather_args(p, C, 1, 1);
+            forward_quads(p, g);
+            g.y = y;
+            if (p->strip) {   // straight into the order that the spread reads
+                g.v_sorted = p->d_ys;
+                g.v_sorted_cpt = cpt;
+            }
+            const int cpl = gather_cpl(g);
+            if ((st = launch(p, PK_GATHER_FWD, s, [&] { return launch_gather(GM_FWD, g, cpl, s); }))) return st;
+        }
+        if ((st = sort_join(p, s)) ||
+            (st = adjoint_impl(p, C, y, (const float2*)smaps, a.q, s, p->strip ? p->d_ys : nullptr)) ||
+            (st = cg(CG_DOT)) || (st = cg(CG_UPDATE)) || (st = cg(CG_DIR)))
+            return st;
+        std::swap(a.rr, a.rr_new);
+    }
+    return finish_call(p, s, NUFFT_OK);
 }
 
 int nufft_get_info(nufft_plan_t p, nufft_plan_info* info) {

@@ -118,6 +118,17 @@ class Plan:
                                _ptr(go, torch.float32, "grad_omega"), _ptr(gx, torch.complex64, "grad_x"), _stream())
         return go, gx
 
+    def cg_normal(self, b, lam, iters, smaps=None):
+        """iters steps of CG, from zero, on (E'E + lam I) x = b, queued as one call (see nufft_cg_normal)."""
+        C = self._coils(b, smaps)
+        x = torch.empty(self._img_shape(C, smaps), dtype=torch.complex64, device=b.device)
+        nbytes = _abi.nufft_cg_work_bytes(self.handle, C, smaps is not None)
+        work = torch.empty(nbytes, dtype=torch.uint8, device=b.device)
+        _abi.nufft_cg_normal(self.handle, C, _ptr(b, torch.complex64, "b", self._img_shape(C, smaps)),
+                             _ptr(smaps, torch.complex64, "smaps", (C,) + self.shape), lam, iters,
+                             _ptr(x, torch.complex64, "x"), _ptr(work, torch.uint8, "work"), nbytes, _stream())
+        return x
+
     def profile_enable(self, enable=True):
         _abi.nufft_profile_enable(self.handle, enable)
 

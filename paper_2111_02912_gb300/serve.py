@@ -33,7 +33,6 @@ import numpy as np
 import torch
 
 from . import _abi
-from .autograd import cg_solve
 from .plan import Plan
 
 
@@ -174,8 +173,7 @@ class Server:
         S = req.smaps
         if req.kind == "recon":
             b = plan.adjoint(req.y, S)
-            F = lambda v: plan.adjoint(plan.forward(v, S), S) + req.lam * v
-            req.result = cg_solve(F, b, req.iters)
+            req.result = plan.cg_normal(b, req.lam, req.iters, S)
         else:   # traj_grad: L = ||E x - y||^2, v = 2 (E x - y)
             v = 2.0 * (plan.forward(req.x, S) - req.y)
             go, _ = plan.vjp_omega_x(req.x, v, S, need_omega=True, need_x=False)
