@@ -96,11 +96,12 @@ typedef struct {
 
 enum { NUFFT_KERNEL_DIRECT = 0, NUFFT_KERNEL_TABLE = 1 };
 
-/* Forward gather (interpolation, Appendix step 3) lane layouts (nufft_opts.gather_variant), all
+/* Gather (interpolation, Appendix step 3) lane layouts (nufft_opts.gather_variant), all
  * computing the same sums: a lane owns two adjacent coils (PAIRS: one 16-byte load per tap) or
- * four (QUADS: one 32-byte load per tap, twice the points per warp; for C a multiple of 4 from 8
- * on, else pairs).  AUTO takes quads for the 2-D forward with C a multiple of 4 from 16 on, where
- * they measured faster, and pairs elsewhere.  The JVP and VJP gathers always use pairs. */
+ * four (QUADS, forward only: one 32-byte load per tap, twice the points per warp; for C a multiple
+ * of 4 from 8 on, else pairs).  AUTO takes, where they measured faster, quads for the 2-D forward
+ * with C a multiple of 4 from 16 on, and for every gather of 8 coils in 2-D and 3-D a layout whose
+ * loads cover whole 128-byte lines of the grid; pairs elsewhere. */
 enum { NUFFT_GATHER_AUTO = 0, NUFFT_GATHER_PAIRS = 1, NUFFT_GATHER_QUADS = 2 };
 
 /* Adjoint spread kernels (nufft_opts.spread_variant), all computing the transpose of the

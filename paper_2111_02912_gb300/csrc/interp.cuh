@@ -240,6 +240,222 @@ __global__ void __launch_bounds__(256, 4) k_gather_occ4(GatherArgs a) {
     gather_body<D, J, ND, CPL, MODE, W>(a);
 }
 
+// Whole-line gather for eight coils.  With 64-byte channel blocks the pair lanes above read eight
+// half lines per warp load, and the L1 data pipe, which serves one line per wavefront, bounds the
+// 3-D gathers (81-83% of its peak at half its bytes).  Here a point has eight lanes, 16 bytes each, and
+// a load covers whole 128-byte lines of the row's cells; lane l always holds coil pair l mod 4.
+//   ND even: a cell is ND / 2 lines; load s of a column reads blocks 2 s (lanes 0-3) and 2 s + 1.
+//   ND odd: two cells, of an even column E and the odd column after it, are ND lines.  The window's
+//   even and odd columns are matched so (one match per row is of two pairs when it starts at an odd
+//   column), and the lines of a match are, for ND = 1: {E0 O0}, and for ND = 3: {E0 E1} {E2 O0} {O1 O2}
+//   (E2 = block 2 of the even column).
+// A load of a match belongs to one channel block and one column per half of the lanes, so each has
+// its own accumulators and its own column weight; the epilogues are linear in the channel blocks, so
+// the halves' partial sums meet only there.  Addresses are 32-bit byte offsets from the grid (the host
+// takes this kernel for grids below 4 GB).
+template <int D, int J, int ND, int MODE>
+__device__ __forceinline__ void gather_lines_body(const GatherArgs& a) {
+    constexpr int CELL = ND * 64;                        // bytes of one cell's channels
+    constexpr bool ODD = ND % 2 == 1;
+    constexpr int S = ODD ? ND : ND / 2;                 // loads per match or column
+    constexpr int NT = ODD ? (J + 1) / 2 : J;            // matches or columns per row
+    extern __shared__ float wsm[];   // [points][D * J]
+    const int tid = threadIdx.x, l = tid & 7;
+    const bool up = l >= 4;          // the upper half of the point's lanes
+    const int64_t pt = (int64_t)blockIdx.x * (blockDim.x >> 3) + (tid >> 3);
+    const bool valid = pt < a.pts.m;
+    float* w = wsm + (tid >> 3) * (D * J);
+    int4 ix = make_int4(0, 0, 0, 0);
+    if (valid) {
+        ix = a.pts.idx[pt];
+        group_weights<D, J>(w, a.pts.w + pt * a.pts.ws, a.pts.wd, l, 8);
+    }
+    __syncwarp();
+    if (!valid) return;
+
+    const int Kl = a.K[D - 1];
+    const int kl0 = D == 2 ? ix.y : ix.z;
+    const float* wc = w + (D - 1) * J;
+    uint32_t off[NT][S];   // byte offset of the lane's 16 bytes within the row
+    float wl[NT][S];       // column weight
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+        if (ODD) {
+            // window positions of the match's even and odd columns; -1: none (J odd)
+            int je = 2 * t, jo = 2 * t + 1 < J ? 2 * t + 1 : -1;
+            if (kl0 & 1) {
+                jo = 2 * t;
+                je = t > 0 ? 2 * t - 1 : (J % 2 == 0 ? J - 1 : -1);
+            }
+            int ce = kl0 + max(je, 0), co = kl0 + max(jo, 0);
+            if (ce >= Kl) ce -= Kl;
+            if (co >= Kl) co -= Kl;
+            const float we = je >= 0 ? wc[max(je, 0)] : 0.f, wo = jo >= 0 ? wc[max(jo, 0)] : 0.f;
+            if (ND == 1) {
+                off[t][0] = (uint32_t)((up ? co : ce) * CELL + (l & 3) * 16);
+                wl[t][0] = up ? wo : we;
+            } else {
+                off[t][0] = (uint32_t)(ce * CELL + l * 16);
+                wl[t][0] = we;
+                off[t][S > 1 ? 1 : 0] = (uint32_t)(up ? co * CELL + (l & 3) * 16 : ce * CELL + 128 + l * 16);
+                wl[t][S > 1 ? 1 : 0] = up ? wo : we;
+                off[t][S - 1] = (uint32_t)(co * CELL + 64 + l * 16);
+                wl[t][S - 1] = wo;
+            }
+        } else {
+            int c = kl0 + t;
+            if (c >= Kl) c -= Kl;
+#pragma unroll
+            for (int i = 0; i < S; ++i) {
+                off[t][i] = (uint32_t)(c * CELL + 128 * i + l * 16);
+                wl[t][i] = wc[t];
+            }
+        }
+    }
+    float4 acc[S];
+#pragma unroll
+    for (int i = 0; i < S; ++i) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+
+    const char* base = (const char*)a.grid;
+    auto row = [&](uint32_t rb, float wr) {
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int i = 0; i < S; ++i) {
+                const float wt = wr * wl[t][i];
+                float4 g;
+                if (ODD && J % 2 == 1 && (t == 0 || t == NT - 1)) {   // the one column that may be missing
+                    g = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (wl[t][i] != 0.f) g = __ldg((const float4*)(base + (rb + off[t][i])));
+                } else {
+                    g = __ldg((const float4*)(base + (rb + off[t][i])));
+                }
+                acc[i].x = fmaf(wt, g.x, acc[i].x);
+                acc[i].y = fmaf(wt, g.y, acc[i].y);
+                acc[i].z = fmaf(wt, g.z, acc[i].z);
+                acc[i].w = fmaf(wt, g.w, acc[i].w);
+            }
+    };
+    const int K0 = a.K[0];
+    if (D == 2) {
+        const uint32_t rstride = (uint32_t)a.K[1] * CELL;
+#pragma unroll
+        for (int j0 = 0; j0 < J; ++j0) {
+            int k0 = ix.x + j0;
+            if (k0 >= K0) k0 -= K0;
+            row((uint32_t)k0 * rstride, w[j0]);
+        }
+    } else {
+        const int K1 = a.K[1];
+        const uint32_t rstride = (uint32_t)a.K[2] * CELL;
+#pragma unroll 1
+        for (int j0 = 0; j0 < J; ++j0) {
+            int k0 = ix.x + j0;
+            if (k0 >= K0) k0 -= K0;
+            const float w0 = w[j0];
+#pragma unroll
+            for (int j1 = 0; j1 < J; ++j1) {
+                int k1 = ix.y + j1;
+                if (k1 >= K1) k1 -= K1;
+                row((uint32_t)(k0 * K1 + k1) * rstride, w0 * w[J + j1]);
+            }
+        }
+    }
+
+    const int64_t orig = ix.w, M = a.M;
+    const unsigned mask = 0xffu << ((tid & 31) & ~7);   // the point's lanes
+    const int c0 = 2 * (l & 3);                         // this lane's coil pair
+    auto block_of = [&](int i) {                        // channel block of load i
+        if (ND == 1) return 0;
+        if (!ODD) return 2 * i + (up ? 1 : 0);
+        return i == 0 ? (up ? 1 : 0) : (i == 1 ? (up ? 0 : 2) : (up ? 2 : 1));
+    };
+    // Sum of what the point's two lanes of a coil pair hold; the lower lane gets the first coil.
+    auto meet = [&](float4 v) {
+        v.x += __shfl_xor_sync(mask, v.x, 4);
+        v.y += __shfl_xor_sync(mask, v.y, 4);
+        v.z += __shfl_xor_sync(mask, v.z, 4);
+        v.w += __shfl_xor_sync(mask, v.w, 4);
+        return up ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
+    };
+    const int c = c0 + (up ? 1 : 0);   // the coil this lane writes
+    if (MODE == GM_FWD || (MODE == GM_JVP && ND > D)) {   // the plain image's values
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < S; ++i)
+            if (block_of(i) == 0) {
+                v.x += acc[i].x;
+                v.y += acc[i].y;
+                v.z += acc[i].z;
+                v.w += acc[i].w;
+            }
+        const float2 y = meet(v);
+        if (MODE == GM_FWD && a.v_sorted_cpt) {   // for the adjoint spread of the same points
+            const int cg = c / a.v_sorted_cpt;
+            a.v_sorted[((int64_t)cg * M + pt) * a.v_sorted_cpt + (c - cg * a.v_sorted_cpt)] = y;
+        } else {
+            a.y[(int64_t)c * M + orig] = y;
+        }
+    }
+    if (MODE == GM_JVP) {   // dy = -i sum_d domega^[d] g_d, the d-th weighted block at d + (plain ? 1 : 0)
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int i = 0; i < S; ++i) {
+            const int d = block_of(i) - (ND > D ? 1 : 0);
+            if (d < 0) continue;
+            const float dom = __ldg(a.domega + (int64_t)d * M + orig);
+            v.x = fmaf(dom, acc[i].y, v.x);
+            v.y = fmaf(-dom, acc[i].x, v.y);
+            v.z = fmaf(dom, acc[i].w, v.z);
+            v.w = fmaf(-dom, acc[i].z, v.w);
+        }
+        a.dy[(int64_t)c * M + orig] = meet(v);
+    }
+    if (MODE == GM_VJP) {
+        const float2 v0 = __ldg(a.v + (int64_t)c0 * M + orig), v1 = __ldg(a.v + (int64_t)(c0 + 1) * M + orig);
+        if (a.v_sorted) {   // for the adjoint spread of the same v
+            const float2 v = up ? v1 : v0;
+            if (a.v_sorted_cpt) {
+                const int cg = c / a.v_sorted_cpt;
+                a.v_sorted[((int64_t)cg * M + pt) * a.v_sorted_cpt + (c - cg * a.v_sorted_cpt)] = v;
+            } else {
+                a.v_sorted[(int64_t)c * M + pt] = v;
+            }
+        }
+        float gsum[D];
+#pragma unroll
+        for (int d = 0; d < D; ++d) gsum[d] = 0.f;
+#pragma unroll
+        for (int i = 0; i < S; ++i) {   // Im{conj(v) g}
+            const float t = (v0.x * acc[i].y - v0.y * acc[i].x) + (v1.x * acc[i].w - v1.y * acc[i].z);
+#pragma unroll
+            for (int d = 0; d < D; ++d) gsum[d] += block_of(i) == d ? t : 0.f;
+        }
+#pragma unroll
+        for (int d = 0; d < D; ++d)
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) gsum[d] += __shfl_xor_sync(mask, gsum[d], o);
+        if (l == 0) {
+#pragma unroll
+            for (int d = 0; d < D; ++d) a.grad[(int64_t)d * M + orig] = gsum[d];
+        }
+    }
+}
+
+// 64-thread blocks (eight points): a block ends as soon as its own points have their taps.  Registers:
+// 96 for three and four channel blocks (20 warps per SM), else 64 (32 warps).
+// 128^2 x 96, 8 coils, 2 M points: VJP 4570 -> 3600 us, forward 1350 -> 1230 us; 128-, 256-, 320- and
+// 640-thread blocks took 3713, 3758, 3761 and 3933 us for the VJP, 80 and 128 registers the same as 96.
+// (32-byte loads by four lanes per point ran no faster than half lines: 5130 us.)  What bounds it now
+// is the latency of the taps' L2 reads: half of them miss L1, 10 TB/s through the crossbar, at 60% of
+// the L1 pipe.
+constexpr int kLinesThreads = 64;
+template <int D, int J, int ND, int MODE>
+__global__ void __launch_bounds__(kLinesThreads, ND >= 3 ? 10 : 16) k_gather_lines(GatherArgs a) {
+    pdl_wait();
+    gather_lines_body<D, J, ND, MODE>(a);
+}
+
 template <int D, int J, int ND, int MODE>
 static cudaError_t gather_cpl(const GatherArgs& a, int cpl, cudaStream_t s) {
     const int threads = 256;
@@ -247,6 +463,14 @@ static cudaError_t gather_cpl(const GatherArgs& a, int cpl, cudaStream_t s) {
     const unsigned blocks = (unsigned)((a.pts.m + gpb - 1) / gpb);
     const size_t smem = (size_t)gpb * D * J * sizeof(float);
     if (blocks == 0) return cudaSuccess;
+    if constexpr (D > 1) {
+        if (cpl == kGatherLines) {
+            const int pts = kLinesThreads / 8;
+            (void)launch_pdl(k_gather_lines<D, J, ND, MODE>, (unsigned)((a.pts.m + pts - 1) / pts), kLinesThreads,
+                             (size_t)pts * D * J * sizeof(float), s, a);
+            return cudaGetLastError();
+        }
+    }
     if (cpl == kGatherQuads) {   // coil quads
         (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 4>, blocks, threads, smem, s, a);
     } else if (cpl == 0) {   // coil pairs
