@@ -291,7 +291,7 @@ inline bool fft2_factor(int L, int& L1, int& L2) {
 cudaError_t launch_sum_chunks(const float2* part, int nparts, int64_t n, float2* x, cudaStream_t s);
 
 // ---------------------------------------------------------- interpolation
-enum GatherMode { GM_FWD = 0, GM_JVP = 1, GM_VJP = 2 };
+enum GatherMode { GM_FWD = 0, GM_JVP = 1, GM_VJP = 2, GM_FWD_SORTED = 3 };
 struct GatherArgs {
     PointsView pts;
     int D, J;
@@ -309,7 +309,7 @@ struct GatherArgs {
     float* grad;          // [D][M]
     float2* v_sorted;     // VJP: if set, v is also written here in sorted point order, [C][M]
     int v_sorted_cpt;     // ... in the strip layout [C / cpt][M][cpt] instead, when > 0
-                          // (forward: with both set, y goes there in the strip layout, not to y)
+                          // (FWD_SORTED: y goes there in the strip layout, not to y)
 };
 // cpl: lane slots per lane (coils l + k G), or 0 for coil pairs, kGatherQuads for coil quads,
 // kGatherLines for whole lines (2-D and 3-D, C = 8)

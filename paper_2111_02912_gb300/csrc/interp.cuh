@@ -7,7 +7,7 @@
 // are evaluated once by the group (one psi per lane) and reused for every
 // channel of every coil: the unweighted grid and the D coordinate-weighted
 // grids x . r^[d] of Eq. (e,Ax).  Epilogues:
-//   FWD  y_c = g_c0
+//   FWD  y_c = g_c0 (FWD_SORTED: in the sorted order that the strip spread reads, 2-D and 3-D)
 //   JVP  dy_c = -i sum_d domega^[d] g_cd  (and y_c when the plain channel is present)
 //   VJP  grad^[d] = sum_c Re{conj(v_c) (-i) g_cd} = sum_c Im{conj(v_c) g_cd}   (Eq. (e,jac,Ax,v))
 // so the D interpolated channels per coil never leave registers.
@@ -157,15 +157,15 @@ __device__ __forceinline__ void gather_body(const GatherArgs& a) {
 #pragma unroll
         for (int k = 0; k < CPL; ++k)
 #pragma unroll
+            for (int i = 0; i < W; ++i)
+                if (ok[k]) a.y[(int64_t)(W * (lane_g + k * G) + i) * M + orig] = acc[0][k][i];
+    } else if (MODE == GM_FWD_SORTED) {   // for the adjoint spread of the same points
+#pragma unroll
+        for (int k = 0; k < CPL; ++k)
+#pragma unroll
             for (int i = 0; i < W; ++i) {
-                if (!ok[k]) continue;
-                const int c = W * (lane_g + k * G) + i;
-                if (a.v_sorted_cpt) {   // for the adjoint spread of the same points
-                    const int cg = c / a.v_sorted_cpt;
-                    a.v_sorted[((int64_t)cg * M + pt) * a.v_sorted_cpt + (c - cg * a.v_sorted_cpt)] = acc[0][k][i];
-                } else {
-                    a.y[(int64_t)c * M + orig] = acc[0][k][i];
-                }
+                const int c = W * (lane_g + k * G) + i, cg = c / a.v_sorted_cpt;
+                if (ok[k]) a.v_sorted[((int64_t)cg * M + pt) * a.v_sorted_cpt + (c - cg * a.v_sorted_cpt)] = acc[0][k][i];
             }
     } else if (MODE == GM_JVP) {
         float dom[D];
@@ -225,17 +225,20 @@ __device__ __forceinline__ void gather_body(const GatherArgs& a) {
     }
 }
 
-template <int D, int J, int ND, int CPL, int MODE, int W>
-__global__ void __launch_bounds__(256) k_gather(GatherArgs a) {
-    pdl_wait();
-    gather_body<D, J, ND, CPL, MODE, W>(a);
+// Block size and resident blocks per SM that the registers are held to (0: no limit).  The gathers wait
+// on their tap loads, so warps count, as long as nothing of weight spills.  Single coils: 64-thread
+// blocks, 64 registers for one and two channel blocks (150 x 218, 5 coils, 30,011 points, VJP: 20.7 ->
+// 15.0 us).  Pairs and quads: 256 threads; the 2-D VJP and JVP pairs are held to four and three blocks
+// (VJP 40.3 -> 39.1 us on the 640^2, 16-coil case; JVP with values, 192 x 256, 12 coils, 99,999 points:
+// 69.6 -> 65.5 us).  The forward at 40 or 48 registers spills and gains nothing.
+constexpr int gather_threads(int W) { return W == 1 ? 64 : 256; }
+constexpr int gather_blocks(int D, int mode, int ND, int CPL, int W) {
+    return W == 1 ? (CPL > 1 ? 8 : ND <= 2 ? 16 : 12)
+           : D == 2 && W == 2 && mode == GM_VJP ? 4
+           : D == 2 && W == 2 && mode == GM_JVP ? 3 : 0;
 }
-
-// The gathers wait on their tap loads.  The 2-D VJP with coil pairs is held to 64 registers (no
-// spill for any J) so that four blocks share an SM: measured 40.3 -> 39.1 us on the 640^2, 16-coil
-// case.  The forward at 40 or 48 registers spills and gains nothing; the other VJP kinds spill at 64.
 template <int D, int J, int ND, int CPL, int MODE, int W>
-__global__ void __launch_bounds__(256, 4) k_gather_occ4(GatherArgs a) {
+__global__ void __launch_bounds__(gather_threads(W), gather_blocks(D, MODE, ND, CPL, W)) k_gather(GatherArgs a) {
     pdl_wait();
     gather_body<D, J, ND, CPL, MODE, W>(a);
 }
@@ -379,7 +382,7 @@ __device__ __forceinline__ void gather_lines_body(const GatherArgs& a) {
         return up ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
     };
     const int c = c0 + (up ? 1 : 0);   // the coil this lane writes
-    if (MODE == GM_FWD || (MODE == GM_JVP && ND > D)) {   // the plain image's values
+    if (MODE == GM_FWD || MODE == GM_FWD_SORTED || (MODE == GM_JVP && ND > D)) {   // the plain image's values
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int i = 0; i < S; ++i)
@@ -390,7 +393,7 @@ __device__ __forceinline__ void gather_lines_body(const GatherArgs& a) {
                 v.w += acc[i].w;
             }
         const float2 y = meet(v);
-        if (MODE == GM_FWD && a.v_sorted_cpt) {   // for the adjoint spread of the same points
+        if (MODE == GM_FWD_SORTED) {   // for the adjoint spread of the same points
             const int cg = c / a.v_sorted_cpt;
             a.v_sorted[((int64_t)cg * M + pt) * a.v_sorted_cpt + (c - cg * a.v_sorted_cpt)] = y;
         } else {
@@ -458,7 +461,7 @@ __global__ void __launch_bounds__(kLinesThreads, ND >= 3 ? 10 : 16) k_gather_lin
 
 template <int D, int J, int ND, int MODE>
 static cudaError_t gather_cpl(const GatherArgs& a, int cpl, cudaStream_t s) {
-    const int threads = 256;
+    const int threads = gather_threads(cpl > 0 ? 1 : 2);
     const int gpb = threads / a.G;
     const unsigned blocks = (unsigned)((a.pts.m + gpb - 1) / gpb);
     const size_t smem = (size_t)gpb * D * J * sizeof(float);
@@ -471,11 +474,11 @@ static cudaError_t gather_cpl(const GatherArgs& a, int cpl, cudaStream_t s) {
             return cudaGetLastError();
         }
     }
-    if (cpl == kGatherQuads) {   // coil quads
-        (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 4>, blocks, threads, smem, s, a);
+    if (cpl == kGatherQuads) {   // coil quads (forward only)
+        if constexpr (MODE == GM_FWD || MODE == GM_FWD_SORTED) (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 4>, blocks, threads, smem, s, a);
+        else return cudaErrorInvalidValue;
     } else if (cpl == 0) {   // coil pairs
-        if constexpr (D == 2 && MODE == GM_VJP) (void)launch_pdl(k_gather_occ4<D, J, ND, 1, MODE, 2>, blocks, threads, smem, s, a);
-        else (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 2>, blocks, threads, smem, s, a);
+        (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 2>, blocks, threads, smem, s, a);
     }
     else if (cpl == 1) (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 1>, blocks, threads, smem, s, a);
     else (void)launch_pdl(k_gather<D, J, ND, 4, MODE, 1>, blocks, threads, smem, s, a);   // C up to 4 G = 128
@@ -485,6 +488,9 @@ static cudaError_t gather_cpl(const GatherArgs& a, int cpl, cudaStream_t s) {
 template <int D, int J>
 static cudaError_t gather_mode(GatherMode mode, const GatherArgs& a, int cpl, cudaStream_t s) {
     if (mode == GM_FWD) return gather_cpl<D, J, 1, GM_FWD>(a, cpl, s);
+    if constexpr (D > 1) {
+        if (mode == GM_FWD_SORTED) return gather_cpl<D, J, 1, GM_FWD_SORTED>(a, cpl, s);
+    }
     if (mode == GM_VJP) return gather_cpl<D, J, D, GM_VJP>(a, cpl, s);
     if (a.nd == D) return gather_cpl<D, J, D, GM_JVP>(a, cpl, s);
     return gather_cpl<D, J, D + 1, GM_JVP>(a, cpl, s);

@@ -1309,7 +1309,8 @@ int nufft_cg_normal(nufft_plan_t p, int C, const nufft_cfloat* b, const nufft_cf
                 g.v_sorted_cpt = cpt;
             }
             const int cpl = gather_cpl(g);
-            if ((st = launch(p, PK_GATHER_FWD, s, [&] { return launch_gather(GM_FWD, g, cpl, s); }))) return st;
+            const GatherMode mode = p->strip ? GM_FWD_SORTED : GM_FWD;
+            if ((st = launch(p, PK_GATHER_FWD, s, [&] { return launch_gather(mode, g, cpl, s); }))) return st;
         }
         if ((st = sort_join(p, s)) ||
             (st = adjoint_impl(p, C, y, (const float2*)smaps, a.q, s, p->strip ? p->d_ys : nullptr)) ||
