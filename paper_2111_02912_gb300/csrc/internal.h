@@ -20,12 +20,14 @@ constexpr int kNbrStride = 64;        // entries per tile in tile_nbr: n, then 2
 // u = (g0 ng1 + g1) nbl + t covers rows g0 R0 .., g1 R1 .. (g1 = 0, R1 = 1 in 2-D) and columns
 // t kStripW .. + kStripW - 1.
 constexpr int kStripW = 16;           // columns of a strip unit (the accumulators of one lane)
+constexpr int kStripLgW = 4;
 // 3-D: rows of a unit along dim 1 for NSL rows in all (R0 = NSL / R1 along dim 0), near square
 __host__ __device__ constexpr int strip_rows1(int nsl) { return nsl >= 32 ? 8 : (nsl >= 8 ? 4 : 2); }
 struct StripGeom {
     int D;
     int K0, K1, KL;     // grid edges: dims 0 and 1, and the last (column) axis (KL = K1 in 2-D)
     int R0, R1;         // rows of a unit along dim 0 and (3-D) dim 1; R1 = 1 in 2-D
+    int lgR0, lgR1;     // their logarithms
     int ng1, nbl;       // row groups along dim 1 (1 in 2-D), column tiles
     int J, NSL;
 };
@@ -33,15 +35,12 @@ struct StripGeom {
 // Distinct groups of R cells (mod K) holding the J cells k .. k + J - 1 of one axis, at most 5:
 // calls f(group, offset) with offset = group start - k (+ K past the wrap), in [-(R-1), J-1].
 template <typename F>
-__device__ __forceinline__ void strip_axis_groups(int k, int K, int R, int J, F f) {
-    int prev = -1;
-    for (int j = 0; j < J; ++j) {
-        int c = k + j;
-        if (c >= K) c -= K;
-        const int grp = c / R;
-        if (grp == prev) continue;
-        prev = grp;
-        f(grp, grp * R - k + (c < k ? K : 0));
+__device__ __forceinline__ void strip_axis_groups(int k, int K, int lg, int J, F f) {
+    for (int j = 0; j < J;) {
+        const int c = k + j < K ? k + j : k + j - K;
+        const int grp = c >> lg, end = min((grp + 1) << lg, K);
+        f(grp, (grp << lg) - k + (c < k ? K : 0));
+        j += end - c;
     }
 }
 
@@ -54,22 +53,15 @@ template <typename F>
 __device__ __forceinline__ void strip_point_units(const StripGeom& g, int4 ix, F unit) {
     const int kl = g.D == 3 ? ix.z : ix.y;
     int tiles[3], sds[3], nt = 0;
-    for (int j = 0; j < g.J; ++j) {
-        int col = kl + j;
-        if (col >= g.KL) col -= g.KL;
-        const int t = col / kStripW;
-        if (nt == 0 || t != tiles[nt - 1]) {
-            if (nt < 3) {
-                tiles[nt] = t;
-                sds[nt] = kl - t * kStripW - (col < kl ? g.KL : 0);   // past the wrap: start lies left
-            }
-            ++nt;
-        }
-    }
-    if (nt > 3) nt = 3;
-    strip_axis_groups(ix.x, g.K0, g.R0, g.J, [&](int g0, int dr0) {
+    strip_axis_groups(kl, g.KL, kStripLgW, g.J, [&](int t, int ofs) {
+        if (nt == 0) { tiles[0] = t; sds[0] = -ofs; }
+        else if (nt == 1) { tiles[1] = t; sds[1] = -ofs; }
+        else { tiles[2] = t; sds[2] = -ofs; }
+        nt = min(nt + 1, 3);
+    });
+    strip_axis_groups(ix.x, g.K0, g.lgR0, g.J, [&](int g0, int dr0) {
         if (g.D == 3) {
-            strip_axis_groups(ix.y, g.K1, g.R1, g.J, [&](int g1, int dr1) {
+            strip_axis_groups(ix.y, g.K1, g.lgR1, g.J, [&](int g1, int dr1) {
                 for (int q = 0; q < nt; ++q) unit((g0 * g.ng1 + g1) * g.nbl + tiles[q], sds[q], dr0, dr1);
             });
         } else {
@@ -85,7 +77,7 @@ __device__ __forceinline__ void strip_point_units(const StripGeom& g, int4 ix, F
 // {unit, first hit, end hit, split index} (split index -1: the unit is one item; else
 // splits[split index] = {part, parts, first partial slot, 0}); the parts of split units come first.
 struct StripTables {
-    int* hcount;      // [nunits]   hits per unit (counted by the scatter; zeroed before it)
+    int* hcount;      // [nunits]   hits per unit (zero before they are counted: 2-D by the scatter, 3-D after it)
     int* hcur;        // [nunits]   fill cursors (zeroed by the plan)
     int* hoff;        // [nunits+1] first hit of each unit
     int2* hits;       // [hit_cap]
@@ -143,10 +135,11 @@ cudaError_t launch_bin_scatter(const SortArgs& a, cudaStream_t s);   // records 
 // Deterministic order: ranks within each bin by original index (before the scatter; tmp is [M]
 // scratch).  Step 0 places the original indices, step 1 ranks them.
 cudaError_t launch_det_ranks(const SortArgs& a, int step, int* tmp, cudaStream_t s);
-// Strip tables (kernels_strip.cu), after the scatter (which counts the hits per unit):
+// Strip tables (kernels_strip.cu), after the scatter (which counts the hits per unit in 2-D):
 cudaError_t launch_strip_plan(const SortArgs& a, int step, cudaStream_t s);   // step 0: block totals; 1: offsets, items
 int strip_plan_blocks(int nunits);   // blocks of the plan launches
 int strip_plan_vals();               // per-block totals the plan keeps
+cudaError_t launch_strip_count(const SortArgs& a, cudaStream_t s);   // 3-D: hits per unit, before the plan
 cudaError_t launch_strip_fill(const SortArgs& a, cudaStream_t s);    // hit lists
 // Deterministic order: the fill writes into hits_tmp, then each unit's hits are ranked by sorted
 // point index into hits.

@@ -37,13 +37,13 @@ int fail(int status, const std::string& msg) {
 enum ProfKind {
     PK_ZERO, PK_BIN_COUNT, PK_BIN_SCAN, PK_TILE_SCAN, PK_BIN_SCATTER, PK_BIN_ITEMS, PK_FFT_FWD_FIRST, PK_FFT_FWD_MID,
     PK_FFT_INV_MID, PK_FFT_INV_LAST, PK_GATHER_FWD, PK_GATHER_JVP, PK_GATHER_VJP, PK_ZERO_HEAVY, PK_SPREAD, PK_SUM_CHUNKS, PK_PERMUTE_Y,
-    PK_STRIP_PLAN_A, PK_STRIP_PLAN_B, PK_STRIP_FILL, PK_DET_PLACE, PK_DET_RANK, PK_STRIP_ORDER, PK_CG, PK_COUNT
+    PK_STRIP_PLAN_A, PK_STRIP_PLAN_B, PK_STRIP_FILL, PK_DET_PLACE, PK_DET_RANK, PK_STRIP_ORDER, PK_CG, PK_STRIP_COUNT, PK_COUNT
 };
 const char* kProfNames[PK_COUNT] = {"zero", "bin_count", "bin_scan", "tile_scan", "bin_scatter", "bin_items", "fft_fwd_first",
                                     "fft_fwd_mid", "fft_inv_mid", "fft_inv_last", "gather_fwd", "gather_jvp",
                                     "gather_vjp", "zero_heavy", "spread", "sum_chunks", "permute_y",
                                     "strip_plan_a", "strip_plan_b", "strip_fill", "det_place", "det_rank",
-                                    "strip_order", "cg"};
+                                    "strip_order", "cg", "strip_count"};
 
 int64_t grid_size(int64_t n, double sigma) {
     int64_t k = (int64_t)std::ceil(sigma * (double)n - 1e-9);
@@ -494,6 +494,8 @@ StripGeom strip_geom(const nufft_plan_s& p) {
     g.KL = (int)p.K[p.D - 1];
     g.R0 = p.SR0;
     g.R1 = p.SR1;
+    g.lgR0 = ilog2(p.SR0);
+    g.lgR1 = ilog2(p.SR1);
     g.ng1 = p.D == 3 ? (int)((p.K[1] + p.SR1 - 1) / p.SR1) : 1;
     g.nbl = (int)((g.KL + kStripW - 1) / kStripW);
     g.J = p.J;
@@ -637,6 +639,7 @@ int sort_rest(nufft_plan_s* p, cudaStream_t s) {
     // they run behind the join event, beside the kernels that read the sorted points, and are
     // joined before the spread or at the end of the call (strip_join).
     if (p->strip) {
+        if (p->D == 3 && (st = launch(p, PK_STRIP_COUNT, ss, [&] { return launch_strip_count(a, ss); }))) return st;
         if ((st = launch(p, PK_STRIP_PLAN_A, ss, [&] { return launch_strip_plan(a, 0, ss); }))) return st;
         if ((st = launch(p, PK_STRIP_PLAN_B, ss, [&] { return launch_strip_plan(a, 1, ss); }))) return st;
         if ((st = launch(p, PK_STRIP_FILL, ss, [&] { return launch_strip_fill(a, ss); }))) return st;
