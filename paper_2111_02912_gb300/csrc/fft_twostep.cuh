@@ -53,9 +53,11 @@ __device__ __forceinline__ void image_row_factors(const ImageSide& im, int64_t b
 // Registers: with L2 = 32 (256-thread blocks of 8 lines) 80 per thread, so that three blocks share
 // an SM (24 warps; the passes are issue- and latency-bound): the register DFTs fit with at most a
 // few bytes of spill (measured on the 640-point passes: FWD_MID 37.6 -> 31.5 us, INV_MID 26.4 ->
-// 22.4 us against 128 registers at two blocks per SM).  Other sizes keep 128: on the 400-point
-// passes (320-thread blocks) 80 registers cost FWD_FIRST 24.5 -> 28.3 us and FWD_MID 17.3 -> 19.0
-// us.  The coil-summing INV_LAST takes 8 coils per block as well when its two chunks add into the
+// 22.4 us against 128 registers at two blocks per SM).  Shorter lines: 72 (L2 = 20, 24) and 64
+// (L2 <= 16); unlimited, FWD_FIRST and INV_LAST took 122-128 registers for loads in flight that a short
+// row does not have (128^2 x 96, 8 coils: FWD_FIRST 408 -> 328 us mean of the 8- and 24-channel
+// launches, INV_LAST 100 -> 68 us; 48 registers gain nothing more and cost the middle passes 6%).
+// The coil-summing INV_LAST takes 8 coils per block as well when its two chunks add into the
 // image (9..16 coils: 640 blocks in 1.4 waves against 320 one-per-SM blocks of 16 coils in 2.1);
 // with more coils it runs 512-thread blocks of 16 at one block per SM.
 // Half-length pruning fixed at compile time (HALF: n_in = L / 2 on the forward side, n_out = L / 2 on
@@ -68,8 +70,10 @@ __host__ __device__ constexpr bool fft2_half_applies() {
     return (KIND == PASS_FWD_FIRST || KIND == PASS_FWD_MID) ? L1 % 4 == 0 : L2 % 4 == 0;
 }
 
+__host__ __device__ constexpr int fft2_regs(int L2) { return L2 == 32 ? 80 : (L2 >= 20 ? 72 : 64); }
+
 template <int L1, int L2, PassKind KIND, bool HALF>
-__global__ void __maxnreg__(L2 != 32 ? 128 : 80) k_line_fft2(LinePass a) {
+__global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
     pdl_wait();
     if (KIND == PASS_INV_MID && a.clear) {   // the image the next pass's two coil chunks add into
         const int64_t nthr = (int64_t)gridDim.x * gridDim.y * blockDim.x;
@@ -131,9 +135,12 @@ __global__ void __maxnreg__(L2 != 32 ? 128 : 80) k_line_fft2(LinePass a) {
             float2* dst = buf + ln * LP;
             if (!FH)   // zero padding (with FH the padded registers are never read)
                 for (int p = h + lane; p < L - h; p += 32) dst[p + p / L2] = make_float2(0.f, 0.f);
-            // image element e sits at position (e - n_in/2) mod L.  A row of up to 384
-            // elements is loaded in one batch of 12 per lane; indices are clamped so the
-            // loads are unconditional and independent (all in flight before the first use).
+            // image element e sits at position (e - n_in/2) mod L.  A row is loaded in
+            // batches of NB elements per lane, one batch for rows of up to 384 elements with
+            // sigma = 2 or 1.25; indices are clamped so the loads are unconditional and
+            // independent (all in flight before the first use).
+            constexpr int NB = FH ? (L / 2 + 31) / 32 < 12 ? (L / 2 + 31) / 32 : 12
+                                  : (L * 4 / 5 + 31) / 32 < 12 ? (L * 4 / 5 + 31) / 32 : 12;
             const int n = a.n_in;
             if (!ok) {
                 for (int e = lane; e < n; e += 32) {
@@ -143,23 +150,23 @@ __global__ void __maxnreg__(L2 != 32 ? 128 : 80) k_line_fft2(LinePass a) {
                 continue;
             }
             const float wgt = kind == Dm1 ? 0.f : (kind >= 0 ? wr : 1.f);   // row factor; last-axis weight below
-            for (int e0 = 0; e0 < n; e0 += 32 * 12) {
-                float2 xv[12], mv[12];
-                float dv[12];
+            for (int e0 = 0; e0 < n; e0 += 32 * NB) {
+                float2 xv[NB], mv[NB];
+                float dv[NB];
 #pragma unroll
-                for (int q = 0; q < 12; ++q) {
+                for (int q = 0; q < NB; ++q) {
                     const int e = min(e0 + q * 32 + lane, n - 1);
                     xv[q] = __ldg(xrow + e);
                     dv[q] = __ldg(deap_last + e);
                 }
                 if (mrow) {
 #pragma unroll
-                    for (int q = 0; q < 12; ++q) mv[q] = __ldg(mrow + min(e0 + q * 32 + lane, n - 1));
+                    for (int q = 0; q < NB; ++q) mv[q] = __ldg(mrow + min(e0 + q * 32 + lane, n - 1));
 #pragma unroll
-                    for (int q = 0; q < 12; ++q) xv[q] = cmul(xv[q], mv[q]);
+                    for (int q = 0; q < NB; ++q) xv[q] = cmul(xv[q], mv[q]);
                 }
 #pragma unroll
-                for (int q = 0; q < 12; ++q) {
+                for (int q = 0; q < NB; ++q) {
                     const int e = e0 + q * 32 + lane;
                     if (e < n) {
                         float sc = rs * dv[q];
@@ -218,12 +225,13 @@ __global__ void __maxnreg__(L2 != 32 ? 128 : 80) k_line_fft2(LinePass a) {
         }
         dft<L1, DIR>(v);
         if (n2 > 0) {
-            const float2* tw = a.ax.tw2 + n2 * L1;   // row n2: exp(-2 pi i n2 k1 / L) at k1
-            sfor<1, L1>([&](auto k1_) {
-                constexpr int k1 = decltype(k1_)::value;
-                float2 w = __ldg(tw + k1);
-                if (DIR > 0) w.y = -w.y;
-                v[k1] = cmul(v[k1], w);
+            // row n2: exp(-2 pi i n2 k1 / L) at k1, read two at a time (L1 is even)
+            const float4* tw = (const float4*)(a.ax.tw2 + n2 * L1);
+            sfor<0, L1 / 2>([&](auto q_) {
+                constexpr int q = decltype(q_)::value;
+                const float4 w = __ldg(tw + q);
+                if constexpr (q > 0) v[2 * q] = DIR > 0 ? cmulc(v[2 * q], make_float2(w.x, w.y)) : cmul(v[2 * q], make_float2(w.x, w.y));
+                v[2 * q + 1] = DIR > 0 ? cmulc(v[2 * q + 1], make_float2(w.z, w.w)) : cmul(v[2 * q + 1], make_float2(w.z, w.w));
             });
         }
         sfor<0, L1>([&](auto k1_) {

@@ -32,7 +32,7 @@ struct StripGeom {
     int J, NSL;
 };
 
-// Distinct groups of R cells (mod K) holding the J cells k .. k + J - 1 of one axis, at most 5:
+// Distinct groups of R = 2^lg cells (mod K) holding the J cells k .. k + J - 1 of one axis, at most 5:
 // calls f(group, offset) with offset = group start - k (+ K past the wrap), in [-(R-1), J-1].
 template <typename F>
 __device__ __forceinline__ void strip_axis_groups(int k, int K, int lg, int J, F f) {
