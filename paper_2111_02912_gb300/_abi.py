@@ -127,7 +127,9 @@ def nufft_plan(opts, m, omega_ptr, stream=0):
 
 
 def nufft_set_points(plan, m, omega_ptr, stream=0):
-    _check(lib().nufft_set_points(plan, int(m), omega_ptr, stream), "nufft_set_points")
+    st = (_lib or lib()).nufft_set_points(plan, int(m), omega_ptr, stream)
+    if st:
+        _check(st, "nufft_set_points")
 
 
 def nufft_sort_points(plan, stream=0):
@@ -135,11 +137,15 @@ def nufft_sort_points(plan, stream=0):
 
 
 def nufft_forward(plan, C, x, smaps, y, stream=0):
-    _check(lib().nufft_forward(plan, int(C), x, smaps, y, stream), "nufft_forward")
+    st = (_lib or lib()).nufft_forward(plan, int(C), x, smaps, y, stream)
+    if st:
+        _check(st, "nufft_forward")
 
 
 def nufft_adjoint(plan, C, y, smaps, x, stream=0):
-    _check(lib().nufft_adjoint(plan, int(C), y, smaps, x, stream), "nufft_adjoint")
+    st = (_lib or lib()).nufft_adjoint(plan, int(C), y, smaps, x, stream)
+    if st:
+        _check(st, "nufft_adjoint")
 
 
 def nufft_jvp_omega(plan, C, x, smaps, domega, dy, y_or_null, stream=0):
@@ -147,7 +153,9 @@ def nufft_jvp_omega(plan, C, x, smaps, domega, dy, y_or_null, stream=0):
 
 
 def nufft_vjp_omega_x(plan, C, x, smaps, v, grad_omega, grad_x, stream=0):
-    _check(lib().nufft_vjp_omega_x(plan, int(C), x, smaps, v, grad_omega, grad_x, stream), "nufft_vjp_omega_x")
+    st = (_lib or lib()).nufft_vjp_omega_x(plan, int(C), x, smaps, v, grad_omega, grad_x, stream)
+    if st:
+        _check(st, "nufft_vjp_omega_x")
 
 
 def nufft_cg_work_bytes(plan, C, has_maps):

@@ -10,8 +10,13 @@ from . import _abi
 
 
 def _ptr(t, dtype, name, shape=None):
+    """Address of a contiguous CUDA tensor of this type (and shape); raises for anything else."""
     if t is None:
         return None
+    # one pass over the conditions for the tensors that satisfy them; the errors are told apart below
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is dtype and t.is_contiguous()
+            and (shape is None or t.shape == shape)):
+        return t.data_ptr()
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError("%s must be a CUDA tensor" % name)
     if t.dtype != dtype:
@@ -23,8 +28,16 @@ def _ptr(t, dtype, name, shape=None):
     return t.data_ptr()
 
 
+# The current stream's handle of the current device, without a Stream object around it: 0.3 against 2.9
+# us, several times a call.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream():
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or _device is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device())
 
 
 class Plan:
@@ -80,10 +93,9 @@ class Plan:
 
     def forward(self, x, smaps=None, out=None):
         C = self._coils(x, smaps)
-        _ptr(x, torch.complex64, "x", self.shape if smaps is not None else None)
+        xp = _ptr(x, torch.complex64, "x", self.shape if smaps is not None else None)
         y = out if out is not None else torch.empty((C, self.M), dtype=torch.complex64, device=x.device)
-        _abi.nufft_forward(self.handle, C, _ptr(x, torch.complex64, "x"),
-                           _ptr(smaps, torch.complex64, "smaps", (C,) + self.shape),
+        _abi.nufft_forward(self.handle, C, xp, _ptr(smaps, torch.complex64, "smaps", (C,) + self.shape),
                            _ptr(y, torch.complex64, "y", (C, self.M)), _stream())
         return y
 
