@@ -70,6 +70,16 @@ __device__ __forceinline__ void strip_point_units(const StripGeom& g, int4 ix, F
     });
 }
 
+// Packed window start of a hit: column sd in [-(J-1), 15] and start-row offsets dr0, dr1 in
+// [-(R-1), J-1] (dr1 = 0 in 2-D).
+__device__ __forceinline__ int strip_meta(int sd, int dr0, int dr1) {
+    return (sd + 8) | ((dr0 + 32) << 8) | ((dr1 + 32) << 16);
+}
+
+constexpr int kPlanLevels = 8;   // part lengths P 2^L that the strip plan may choose from
+// Parts of 2^lgP hits in a unit of h.
+__device__ __forceinline__ int plan_parts(int h, int lgP) { return max(1, (int)(((int64_t)h + (1 << lgP) - 1) >> lgP)); }
+
 // Sort-time tables of the strip spread (once per omega, read by every adjoint of those points).
 // A hit is a point whose window reaches a unit: {sorted point index, packed window start}, the
 // start column relative to the unit in bits 0..7 (biased by 8) and the start-row offsets along
@@ -125,6 +135,8 @@ struct SortArgs {
     StripTables st;
 };
 cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t s);
+// The whole sort of a strip plan in one launch, for few points (clear: zero the counts first).
+cudaError_t launch_sort_small(const SortArgs& a, bool clear, cudaStream_t s);
 cudaError_t launch_key_count(const SortArgs& a, cudaStream_t s);     // histogram of bins, rank within bin
 cudaError_t launch_bin_scan(const SortArgs& a, cudaStream_t s);      // offsets; clears the histogram
 cudaError_t launch_tile_lists(const SortArgs& a, cudaStream_t s);    // reaching bins, parts per tile

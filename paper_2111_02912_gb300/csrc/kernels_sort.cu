@@ -65,9 +65,8 @@ __global__ void k_zero(float4* p, int64_t n4, int* tail, int64_t ntail) {
 // (a trajectory's readout) usually share a bin, so the lanes of a warp with the
 // same bin take one atomic between them: the group leader adds the group size
 // and the others offset from the returned base by their rank in the group.
-__global__ void k_key_count(SortArgs a) {
-    pdl_wait();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// Called by whole warps, i consecutive over the lanes.
+__device__ __forceinline__ void count_point(const SortArgs& a, int64_t i) {
     const bool live = i < a.m;
     int key = -1;
     if (live) {
@@ -87,6 +86,11 @@ __global__ void k_key_count(SortArgs a) {
     base = __shfl_sync(peers, base, leader);
     a.keyid[i] = key;
     a.local[i] = base + rank;
+}
+
+__global__ void k_key_count(SortArgs a) {
+    pdl_wait();
+    count_point(a, (int64_t)blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 // Block-wide exclusive scan of one value per thread; returns the block total.
@@ -252,15 +256,14 @@ cudaError_t launch_det_ranks(const SortArgs& a, int step, int* tmp, cudaStream_t
     return cudaGetLastError();
 }
 
-__global__ void k_bin_scatter(SortArgs a) {
-    pdl_wait();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= a.m) return;
+// The record and weights of point i at its sorted position (offsets by L2 loads: in the one-launch
+// sort another block of the cluster wrote them).
+__device__ __forceinline__ int4 scatter_point(const SortArgs& a, int64_t i) {
     int4 ix;
     float4 fr;
     int64_t key;
     point_record(a, i, ix, fr, key);
-    const int dst = a.offsets[a.keyid[i]] + a.local[i];
+    const int dst = __ldcg(a.offsets + a.keyid[i]) + a.local[i];
     a.local[i] = dst;   // the inverse of the sort permutation, for reordering coil values
     a.pidx[dst] = ix;
     a.pfrac[dst] = fr;
@@ -274,8 +277,139 @@ __global__ void k_bin_scatter(SortArgs a) {
             for (int j = 0; j < a.J; ++j) w[d * a.wd + j] = kb_psi(a.kb.a, a.kb.two_over_j, u0 - (float)j);
         for (int j = a.J; j < a.wd; ++j) w[d * a.wd + j] = 0.f;
     }
+    return ix;
+}
+
+__global__ void k_bin_scatter(SortArgs a) {
+    pdl_wait();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= a.m) return;
+    const int4 ix = scatter_point(a, i);
     // 2-D strips: count the point as a hit of every unit its window reaches (3-D: k_strip_hits)
     if (a.strip && a.D == 2) strip_point_units(a.sg, ix, [&](int u, int, int, int) { atomicAdd(a.st.hcount + u, 1); });
+}
+
+// The whole sort of a strip plan in one launch, for few points: histogram, bin scan, scatter with the
+// hit counts, strip plan and hit lists as phases of one cluster of eight blocks, a cluster barrier
+// between two of them; the scans and the plan run in block 0.  Separate launches spend 3 to 5 us each
+// on this much work, and the host 1.5 us: 40^2,
+// 80 points: six launches of 31 us in all -> 19 us; 64^2, 4096 points: 30 -> 28 us, five launches
+// fewer.  At 30,011 points it took 107 us for 40: one point per thread is the limit.
+constexpr int kSmallBlocks = 8, kSmallThreads = 512;
+
+__global__ void __launch_bounds__(kSmallThreads, 1) k_sort_small(SortArgs a, int clear) {
+    pdl_wait();
+    __shared__ int sh[32];
+    __shared__ int s_parts[kPlanLevels];
+    const StripTables& T = a.st;
+    const int t = threadIdx.x, g = (int)blockIdx.x * kSmallThreads + t;
+    constexpr int NT = kSmallBlocks * kSmallThreads;
+    if (clear) {   // the counts of a new plan, or of a sort in a graph
+        for (int k = g; k < a.nbins; k += NT) a.kcount[k] = 0;
+        for (int k = g; k < a.nunits; k += NT) T.hcount[k] = 0;
+        cluster_barrier();
+    }
+    const int64_t mpad = (a.m + 31) & ~(int64_t)31;   // whole warps
+    for (int64_t i = g; i < mpad; i += NT) count_point(a, i);
+    cluster_barrier();
+    if (blockIdx.x == 0) {   // bin offsets; the histogram is cleared on the way
+        const int per = (a.nbins + kSmallThreads - 1) / kSmallThreads;
+        const int lo = min(a.nbins, t * per), hi = min(a.nbins, lo + per);
+        int s = 0, excl;
+        for (int b = lo; b < hi; ++b) s += __ldcg(a.kcount + b);
+        block_exclusive_scan(s, sh, excl);
+        for (int b = lo; b < hi; ++b) {
+            const int v = __ldcg(a.kcount + b);
+            a.offsets[b] = excl;
+            a.kcount[b] = 0;
+            excl += v;
+        }
+        if (t == 0) {
+            a.offsets[a.nbins] = (int)a.m;
+            a.heavy[0] = 0;
+        }
+    }
+    cluster_barrier();
+    for (int64_t i = g; i < a.m; i += NT) {
+        const int4 ix = scatter_point(a, i);
+        strip_point_units(a.sg, ix, [&](int u, int, int, int) { atomicAdd(T.hcount + u, 1); });
+    }
+    cluster_barrier();
+    if (blockIdx.x == 0) {   // the strip plan (k_strip_plan_a and _b for one block)
+        const int per = (a.nunits + kSmallThreads - 1) / kSmallThreads;
+        const int lo = min(a.nunits, t * per), hi = min(a.nunits, lo + per);
+        const int lgP0 = 31 - __clz(T.P);
+        if (t < kPlanLevels) s_parts[t] = 0;
+        __syncthreads();
+        int hits = 0, np[kPlanLevels];
+#pragma unroll
+        for (int L = 0; L < kPlanLevels; ++L) np[L] = 0;
+        for (int u = lo; u < hi; ++u) {
+            const int h = __ldcg(T.hcount + u);
+            hits += h;
+#pragma unroll
+            for (int L = 0; L < kPlanLevels; ++L) {
+                const int parts = plan_parts(h, lgP0 + L);
+                if (parts > 1) np[L] += parts;
+            }
+        }
+#pragma unroll
+        for (int L = 0; L < kPlanLevels; ++L) {
+            const int x = __reduce_add_sync(0xffffffffu, np[L]);
+            if ((t & 31) == 0 && x) atomicAdd(&s_parts[L], x);
+        }
+        __syncthreads();
+        int L = 0;
+        while (L < kPlanLevels - 1 && s_parts[L] > T.slots) ++L;
+        const bool fits = s_parts[L] <= T.slots;
+        const int lgP = lgP0 + L, H = fits ? s_parts[L] : 0;
+        int my_parts = 0, my_whole = 0;
+        for (int u = lo; u < hi; ++u) {
+            const int parts = fits ? plan_parts(__ldcg(T.hcount + u), lgP) : 1;
+            if (parts > 1) my_parts += parts;
+            else ++my_whole;
+        }
+        int eh, ep, ew;
+        block_exclusive_scan(hits, sh, eh);
+        block_exclusive_scan(my_parts, sh, ep);
+        const int whole = block_exclusive_scan(my_whole, sh, ew);
+        for (int u = lo; u < hi; ++u) {
+            const int h = __ldcg(T.hcount + u), parts = fits ? plan_parts(h, lgP) : 1;
+            T.hoff[u] = eh;
+            T.hcount[u] = 0;
+            T.hcur[u] = 0;
+            if (parts > 1) {
+                const int slot0 = ep;
+                for (int k = 0; k < parts; ++k, ++ep) {
+                    const int hb = eh + (k << lgP);
+                    T.items[ep] = make_int4(u, hb, min(hb + (1 << lgP), eh + h), ep);
+                    T.splits[ep] = make_int4(k, parts, slot0, 0);
+                }
+            } else {
+                T.items[H + ew] = make_int4(u, eh, eh + h, -1);
+                ++ew;
+            }
+            eh += h;
+        }
+        if (t == kSmallThreads - 1) T.hoff[a.nunits] = eh;
+        if (t == 0) {
+            T.nitems[0] = H + whole;
+            T.nitems[1] = 1 << lgP;
+        }
+    }
+    cluster_barrier();
+    for (int64_t p = g; p < a.m; p += NT) {   // hit lists, as k_strip_fill
+        const int4 ix = __ldcg(a.pidx + p);
+        strip_point_units(a.sg, ix, [&](int u, int sd, int dr0, int dr1) {
+            const int64_t pos = (int64_t)__ldcg(T.hoff + u) + atomicAdd(T.hcur + u, 1);
+            if (pos < T.hit_cap) T.fill_to[pos] = make_int2((int)p, strip_meta(sd, dr0, dr1));
+        });
+    }
+}
+
+cudaError_t launch_sort_small(const SortArgs& a, bool clear, cudaStream_t s) {
+    (void)launch_pdl_cluster(k_sort_small, kSmallBlocks, kSmallThreads, s, a, clear ? 1 : 0);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_zero(void* p, size_t bytes, cudaStream_t s) {

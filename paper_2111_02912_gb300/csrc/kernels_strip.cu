@@ -102,12 +102,6 @@ __device__ __forceinline__ void block_scan_tiles(int n, int (&carry)[V], Get get
 }
 
 // --------------------------------------------------------------- sort tables
-// Packed window start of a hit: column sd in [-(J-1), 15] and start-row offsets dr0, dr1 in
-// [-(R-1), J-1] (dr1 = 0 in 2-D).
-__device__ __forceinline__ int strip_meta(int sd, int dr0, int dr1) {
-    return (sd + 8) | ((dr0 + 32) << 8) | ((dr1 + 32) << 16);
-}
-
 // The plan in two launches of 256-thread blocks (unit b * 256 + t in block b, thread t).  Split
 // parts are counted for P * 2^L, L = 0..7: the smallest level whose split parts fit the partial
 // slots is used.  (a) Per block and level: hits, split parts and whole units.  (b) Every block sums
@@ -115,10 +109,8 @@ __device__ __forceinline__ int strip_meta(int sd, int dr0, int dr1) {
 // offsets and items (split parts first: they start in the first wave), clearing the hit counts
 // (the next sort's scatter counts into them) and the fill cursors.
 constexpr int kPlanThreads = 256;
-constexpr int kPlanLevels = 8;
 constexpr int kPlanVals = 1 + 2 * kPlanLevels;   // hits, then split parts and whole units per level
 
-__device__ __forceinline__ int plan_parts(int h, int lgP) { return max(1, (int)(((int64_t)h + (1 << lgP) - 1) >> lgP)); }
 
 __global__ void __launch_bounds__(kPlanThreads) k_strip_plan_a(SortArgs a) {
     pdl_wait();

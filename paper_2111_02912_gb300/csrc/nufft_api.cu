@@ -37,13 +37,14 @@ int fail(int status, const std::string& msg) {
 enum ProfKind {
     PK_ZERO, PK_BIN_COUNT, PK_BIN_SCAN, PK_TILE_SCAN, PK_BIN_SCATTER, PK_BIN_ITEMS, PK_FFT_FWD_FIRST, PK_FFT_FWD_MID,
     PK_FFT_INV_MID, PK_FFT_INV_LAST, PK_GATHER_FWD, PK_GATHER_JVP, PK_GATHER_VJP, PK_ZERO_HEAVY, PK_SPREAD, PK_SUM_CHUNKS, PK_PERMUTE_Y,
-    PK_STRIP_PLAN_A, PK_STRIP_PLAN_B, PK_STRIP_FILL, PK_DET_PLACE, PK_DET_RANK, PK_STRIP_ORDER, PK_CG, PK_STRIP_COUNT, PK_COUNT
+    PK_STRIP_PLAN_A, PK_STRIP_PLAN_B, PK_STRIP_FILL, PK_DET_PLACE, PK_DET_RANK, PK_STRIP_ORDER, PK_CG, PK_STRIP_COUNT, PK_SORT_SMALL, PK_COUNT
 };
 const char* kProfNames[PK_COUNT] = {"zero", "bin_count", "bin_scan", "tile_scan", "bin_scatter", "bin_items", "fft_fwd_first",
                                     "fft_fwd_mid", "fft_inv_mid", "fft_inv_last", "gather_fwd", "gather_jvp",
                                     "gather_vjp", "zero_heavy", "spread", "sum_chunks", "permute_y",
                                     "strip_plan_a", "strip_plan_b", "strip_fill", "det_place", "det_rank",
-                                    "strip_order", "cg", "strip_count"};
+                                    "strip_order", "cg", "strip_count",
+                                    "sort_small"};
 
 int64_t grid_size(int64_t n, double sigma) {
     int64_t k = (int64_t)std::ceil(sigma * (double)n - 1e-9);
@@ -546,6 +547,11 @@ SortArgs sort_args(nufft_plan_s* p, const float* omega) {
 
 int sort_rest(nufft_plan_s* p, cudaStream_t s);
 
+// The one-launch sort runs up to this many points (one per thread of its cluster), and bins and strip
+// units (which one block scans).
+constexpr int64_t kSmallSortPoints = 4096;
+constexpr int kSmallSortTables = 16384;
+
 // True, with the capture sequence id, when s is recording into a CUDA graph.
 bool capture_id(cudaStream_t s, unsigned long long& id) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -607,6 +613,17 @@ int sort_rest(nufft_plan_s* p, cudaStream_t s) {
         ss = p->aux;
     }
     int st;
+    if (p->strip && !p->deterministic && p->M > 0 && p->M <= kSmallSortPoints && p->nbins <= kSmallSortTables &&
+        p->nunits <= kSmallSortTables) {
+        const bool clear = capturing || !p->kcount_clear;
+        if ((st = launch(p, PK_SORT_SMALL, ss, [&] { return launch_sort_small(a, clear, ss); }))) return st;
+        if (!capturing) p->kcount_clear = true;
+        if (p->aux) {   // records and strip tables are ready together
+            NJ_CUDA(cudaEventRecord(p->join_ev, p->aux));
+            p->join_pending = true;
+        }
+        return NUFFT_OK;
+    }
     // every scan leaves the histogram zero for the next sort; a fresh one, or one in a graph, is cleared
     if ((capturing || !p->kcount_clear) &&
         (st = launch(p, PK_ZERO, ss, [&] { return launch_zero(p->d_kcount, sizeof(int) * sort_keys(*p), ss); })))
