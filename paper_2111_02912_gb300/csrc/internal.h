@@ -76,7 +76,7 @@ __device__ __forceinline__ int strip_meta(int sd, int dr0, int dr1) {
     return (sd + 8) | ((dr0 + 32) << 8) | ((dr1 + 32) << 16);
 }
 
-constexpr int kPlanLevels = 8;   // part lengths P 2^L that the strip plan may choose from
+constexpr int kPlanLevels = 12;  // part lengths P 2^L that the strip plan may choose from
 // Parts of 2^lgP hits in a unit of h.
 __device__ __forceinline__ int plan_parts(int h, int lgP) { return max(1, (int)(((int64_t)h + (1 << lgP) - 1) >> lgP)); }
 

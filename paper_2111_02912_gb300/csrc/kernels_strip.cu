@@ -103,7 +103,7 @@ __device__ __forceinline__ void block_scan_tiles(int n, int (&carry)[V], Get get
 
 // --------------------------------------------------------------- sort tables
 // The plan in two launches of 256-thread blocks (unit b * 256 + t in block b, thread t).  Split
-// parts are counted for P * 2^L, L = 0..7: the smallest level whose split parts fit the partial
+// parts are counted for P * 2^L, L = 0..11: the smallest level whose split parts fit the partial
 // slots is used.  (a) Per block and level: hits, split parts and whole units.  (b) Every block sums
 // the totals of the blocks before it, picks the level, scans its own units and writes their hit
 // offsets and items (split parts first: they start in the first wave), clearing the hit counts

@@ -93,7 +93,7 @@ struct nufft_plan_s {
     int gather_variant = NUFFT_GATHER_AUTO;
     float* d_kbtab = nullptr;      // [tab_n + 2] psi(l / tab_L), zero from tab_n on
     int2* d_hits_tmp = nullptr;    // [hit_cap] the fill's list before ordering (deterministic only)
-    int NSL = 2, SR0 = 2, SR1 = 1, nunits = 0, strip_P = 64, strip_slots = 0, ncg_max = 1;
+    int NSL = 2, SR0 = 2, SR1 = 1, nunits = 0, strip_P = 32, strip_slots = 0, ncg_max = 1;
     float2* d_ys = nullptr;        // [ncg_max][M_cap][64 / NSL] coil values in sorted point order
     float2* d_partial = nullptr;   // [strip_slots][ncg_max][kStripW][32] coil pairs (float4)
     int* d_counters = nullptr;     // [strip_slots][ncg_max], zero between calls
@@ -338,9 +338,6 @@ int validate_opts(const nufft_opts* o, nufft_plan_s& p) {
             if (p.D == 3) nu *= (p.K[1] + p.SR1 - 1) / p.SR1;
             if (nu >= ((int64_t)1 << 30)) return fail(NUFFT_ERR_UNSUPPORTED, "too many strip units");
             p.nunits = (int)nu;
-            // partial-sum slots for split units (8 KB each): ~nunits / 4, at most 16 MB (the plan
-            // lengthens the parts of split units when they would need more)
-            p.strip_slots = std::max(64, std::min(2048 / p.ncg_max, p.nunits / 4));
         }
     }
     // KB power-series coefficients a_k = (beta^2/4)^k / (k!)^2
@@ -400,6 +397,20 @@ void workspace_elems(const nufft_plan_s& p, size_t& G, size_t& T) {
     G = std::max<size_t>(G, (size_t)(p.maxC * p.Nimg));
 }
 
+// Sort histogram entries: one per bin.
+int64_t sort_keys(const nufft_plan_s& p) { return (int64_t)p.nbins; }
+
+// Partial-sum slots for the parts of split units (8 KB per slot and coil group): one per unit, at most one
+// per 24 points, at least 256 of both, and at most 64 MB in all; the sort lengthens the parts when they would
+// need more, which leaves the heaviest warps with long serial sums.  With a quarter of a slot per unit, 16 MB
+// in all and parts of 64 hits the spread took 43 us at 256^2, 4 coils, 65,537 points (now 32), 24 at 64^2,
+// 1 coil, 4096 points (17), 147 at 384^2, 32 coils, 200,000 points (133), 2170 at 128^2 x 96, 8 coils, 2 M
+// points (1985) and 590 at 90 x 100 x 70, 6 coils, 500,003 points (507).
+int strip_slots_for(const nufft_plan_s& p, int64_t cap) {
+    const int64_t n = std::min<int64_t>(std::max<int64_t>(256, cap / 24), std::max(256, p.nunits));
+    return (int)std::max<int64_t>(64, std::min<int64_t>(n, 8192 / p.ncg_max));
+}
+
 // Upper bound of the spread work items: one per tile plus one per P candidates;
 // every point is a candidate of at most 3^D tiles.
 size_t max_items(const nufft_plan_s& p, int64_t cap) {
@@ -407,16 +418,13 @@ size_t max_items(const nufft_plan_s& p, int64_t cap) {
     for (int d = 0; d < p.D; ++d) nbr *= std::min(3, p.nb[d]);
     size_t n = (size_t)p.nbins + (size_t)((nbr * cap + p.P - 1) / p.P) + 1;
     // strips: one item per unit, plus the extra parts of split units (at most the partial slots)
-    if (p.strip) n = std::max(n, (size_t)p.nunits + (size_t)p.strip_slots + 1);
+    if (p.strip) n = std::max(n, (size_t)p.nunits + (size_t)strip_slots_for(p, cap) + 1);
     return n;
 }
 
-// Sort histogram entries: one per bin.
-int64_t sort_keys(const nufft_plan_s& p) { return (int64_t)p.nbins; }
-
-size_t strip_bytes(const nufft_plan_s& p) {
+size_t strip_bytes(const nufft_plan_s& p, int64_t cap) {
     if (!p.strip) return 0;
-    return (size_t)p.strip_slots * (p.ncg_max * (kStripW * 32 * sizeof(float4) + sizeof(int)) + sizeof(int4)) +
+    return (size_t)strip_slots_for(p, cap) * (p.ncg_max * (kStripW * 32 * sizeof(float4) + sizeof(int)) + sizeof(int4)) +
            (size_t)(3 * p.nunits + 3) * sizeof(int);
 }
 
@@ -446,6 +454,10 @@ int alloc_points(nufft_plan_s* p, int64_t cap) {
     p->d_ys = nullptr;
     p->d_hits = nullptr;
     p->d_hits_tmp = nullptr;
+    cudaFree(p->d_partial); cudaFree(p->d_counters); cudaFree(p->d_splits);
+    p->d_partial = nullptr;
+    p->d_counters = nullptr;
+    p->d_splits = nullptr;
     const size_t c = (size_t)std::max<int64_t>(cap, 1);
     if (p->strip) {
         p->hit_cap = (int64_t)c * strip_hits_per_point(*p);
@@ -455,6 +467,17 @@ int alloc_points(nufft_plan_s* p, int64_t cap) {
             cudaGetLastError();
             return fail(NUFFT_ERR_OOM, "device allocation of the strip hit lists failed");
         }
+        p->strip_slots = strip_slots_for(*p, cap);
+        const size_t nslot = (size_t)p->strip_slots * p->ncg_max;
+        if (cudaMalloc(&p->d_partial, nslot * kStripW * 32 * sizeof(float4)) != cudaSuccess ||
+            cudaMalloc(&p->d_counters, nslot * sizeof(int)) != cudaSuccess ||
+            cudaMalloc(&p->d_splits, (size_t)p->strip_slots * sizeof(int4)) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(NUFFT_ERR_OOM, "device allocation of the strip partial sums failed");
+        }
+        // done before any stream of the caller's or the plan's uses them
+        if (cudaMemset(p->d_counters, 0, nslot * sizeof(int)) != cudaSuccess || cudaStreamSynchronize(nullptr) != cudaSuccess)
+            return fail(NUFFT_ERR_CUDA, "clearing the strip counters failed");
     }
     if (cudaMalloc(&p->d_items, max_items(*p, cap) * sizeof(int4)) != cudaSuccess ||
         cudaMalloc(&p->d_local, c * sizeof(int)) != cudaSuccess ||
@@ -1060,7 +1083,7 @@ size_t nufft_workspace_bytes(const nufft_opts* o, int64_t m, int C) {
     size_t G, T;
     workspace_elems(p, G, T);
     size_t b = (G + T) * sizeof(float2) + point_bytes(p, std::max<int64_t>(m, 1));
-    b += (size_t)((4 + kNbrStride) * p.nbins + 2 * sort_keys(p) + 8) * sizeof(int) + strip_bytes(p);
+    b += (size_t)((4 + kNbrStride) * p.nbins + 2 * sort_keys(p) + 8) * sizeof(int) + strip_bytes(p, std::max<int64_t>(m, 1));
     for (int d = 0; d < p.D; ++d) b += (size_t)p.N[d] * sizeof(float) + 2 * (size_t)p.K[d] * sizeof(float2);
     if (p.kernel_mode == NUFFT_KERNEL_TABLE) b += (size_t)(p.tab_n + 2) * sizeof(float);
     return b;
@@ -1120,17 +1143,12 @@ int nufft_plan(nufft_plan_t* out, const nufft_opts* o, int64_t m, const float* o
         return oom("bins");
     cudaMemset(p->d_nitems, 0, 2 * sizeof(int));
     if (p->strip) {
-        const size_t nslot = (size_t)p->strip_slots * p->ncg_max;
-        if (cudaMalloc(&p->d_partial, nslot * kStripW * 32 * sizeof(float4)) != cudaSuccess ||
-            cudaMalloc(&p->d_counters, nslot * sizeof(int)) != cudaSuccess ||
-            cudaMalloc(&p->d_hcount, (size_t)p->nunits * sizeof(int)) != cudaSuccess ||
+        if (cudaMalloc(&p->d_hcount, (size_t)p->nunits * sizeof(int)) != cudaSuccess ||
             cudaMalloc(&p->d_hcur, (size_t)p->nunits * sizeof(int)) != cudaSuccess ||
             cudaMalloc(&p->d_plan_sums, (size_t)strip_plan_blocks(p->nunits) * strip_plan_vals() * sizeof(int)) !=
                 cudaSuccess ||
-            cudaMalloc(&p->d_hoff, (size_t)(p->nunits + 1) * sizeof(int)) != cudaSuccess ||
-            cudaMalloc(&p->d_splits, (size_t)p->strip_slots * sizeof(int4)) != cudaSuccess)
-            return oom("strip partial sums");
-        cudaMemset(p->d_counters, 0, nslot * sizeof(int));
+            cudaMalloc(&p->d_hoff, (size_t)(p->nunits + 1) * sizeof(int)) != cudaSuccess)
+            return oom("strip units");
         cudaMemset(p->d_hcount, 0, (size_t)p->nunits * sizeof(int));
     }
     workspace_elems(*p, p->G_elems, p->T_elems);
@@ -1360,7 +1378,7 @@ int nufft_get_info(nufft_plan_t p, nufft_plan_info* info) {
     info->m = p->M;
     info->nbins = p->nbins;
     info->max_coils = p->maxC;
-    info->workspace_bytes = (p->G_elems + p->T_elems) * sizeof(float2) + point_bytes(*p, p->M_cap) + strip_bytes(*p);
+    info->workspace_bytes = (p->G_elems + p->T_elems) * sizeof(float2) + point_bytes(*p, p->M_cap) + strip_bytes(*p, p->M_cap);
     return NUFFT_OK;
 }
 
