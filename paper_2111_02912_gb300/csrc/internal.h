@@ -131,6 +131,7 @@ struct SortArgs {
     int tab_n;
     // strip mode: the scatter also counts the strip units' hits, then the plan and fill
     int strip, nunits;
+    int hash_hits;        // strips: hits counted and listed by k_strip_hits, not by the scatter and k_strip_fill
     StripGeom sg;
     StripTables st;
 };

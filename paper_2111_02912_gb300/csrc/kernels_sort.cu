@@ -286,7 +286,7 @@ __global__ void k_bin_scatter(SortArgs a) {
     if (i >= a.m) return;
     const int4 ix = scatter_point(a, i);
     // 2-D strips: count the point as a hit of every unit its window reaches (3-D: k_strip_hits)
-    if (a.strip && a.D == 2) strip_point_units(a.sg, ix, [&](int u, int, int, int) { atomicAdd(a.st.hcount + u, 1); });
+    if (a.strip && !a.hash_hits) strip_point_units(a.sg, ix, [&](int u, int, int, int) { atomicAdd(a.st.hcount + u, 1); });
 }
 
 // The whole sort of a strip plan in one launch, for few points: histogram, bin scan, scatter with the

@@ -321,7 +321,7 @@ int strip_plan_vals() { return kPlanVals; }
 
 cudaError_t launch_strip_fill(const SortArgs& a, cudaStream_t s) {
     if (a.m == 0) return cudaSuccess;
-    if (a.D == 3) (void)launch_pdl(k_strip_hits<true>, (unsigned)((a.m + kHitThreads - 1) / kHitThreads), kHitThreads, 0, s, a);
+    if (a.hash_hits) (void)launch_pdl(k_strip_hits<true>, (unsigned)((a.m + kHitThreads - 1) / kHitThreads), kHitThreads, 0, s, a);
     else (void)launch_pdl(k_strip_fill, (unsigned)((a.m + 255) / 256), 256, 0, s, a);
     return cudaGetLastError();
 }

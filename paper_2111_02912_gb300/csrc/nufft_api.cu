@@ -527,6 +527,11 @@ StripGeom strip_geom(const nufft_plan_s& p) {
     return g;
 }
 
+// From this many points the hits of 2-D strips are collected per block too (kernels_strip.cu): 384^2, 32
+// coils, 200,000 points: scatter 34.5 -> 25.7 us, fill 35.2 -> 16.2, count 14.9, the step 806 -> 789; at 51,200
+// points the extra launch costs what it gains (191.3 -> 191.0).  3-D: always.
+constexpr int64_t kHashHitPoints = 100000;
+
 SortArgs sort_args(nufft_plan_s* p, const float* omega) {
     SortArgs a{};
     a.omega = omega;
@@ -562,6 +567,7 @@ SortArgs sort_args(nufft_plan_s* p, const float* omega) {
     a.tab_L = (float)p->tab_L;
     a.tab_n = p->tab_n;
     a.strip = p->strip ? 1 : 0;
+    a.hash_hits = p->strip && (p->D == 3 || p->M >= kHashHitPoints) ? 1 : 0;
     a.nunits = p->nunits;
     a.sg = strip_geom(*p);
     a.st = strip_tables(*p);
@@ -679,7 +685,7 @@ int sort_rest(nufft_plan_s* p, cudaStream_t s) {
     // they run behind the join event, beside the kernels that read the sorted points, and are
     // joined before the spread or at the end of the call (strip_join).
     if (p->strip) {
-        if (p->D == 3 && (st = launch(p, PK_STRIP_COUNT, ss, [&] { return launch_strip_count(a, ss); }))) return st;
+        if (a.hash_hits && (st = launch(p, PK_STRIP_COUNT, ss, [&] { return launch_strip_count(a, ss); }))) return st;
         if ((st = launch(p, PK_STRIP_PLAN_A, ss, [&] { return launch_strip_plan(a, 0, ss); }))) return st;
         if ((st = launch(p, PK_STRIP_PLAN_B, ss, [&] { return launch_strip_plan(a, 1, ss); }))) return st;
         if ((st = launch(p, PK_STRIP_FILL, ss, [&] { return launch_strip_fill(a, ss); }))) return st;
