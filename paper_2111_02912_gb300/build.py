@@ -11,6 +11,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libnufftjac.so")
 SOURCES = ["kernels_fft2_fwd_mid.cu", "kernels_fft2_fwd_first.cu", "kernels_fft2_inv_mid.cu", "kernels_fft2_inv_last.cu",
+           "kernels_fft2_fwd_midb.cu", "kernels_fft2_fwd_firstb.cu", "kernels_fft2_inv_midb.cu", "kernels_fft2_inv_lastb.cu",
            "kernels_gather_d3.cu", "kernels_gather_d2.cu", "kernels_gather_d1.cu", "nufft_api.cu", "kernels_sort.cu",
            "kernels_fft.cu", "kernels_spread.cu", "kernels_strip.cu", "kernels_cg.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -13,8 +13,8 @@
 // the L2 values of row k1, takes the L2-point DFT and writes X[k1 + L1 k2].
 // Consecutive threads work on consecutive lines (the lines of a tile are
 // adjacent in memory), so global loads and stores are coalesced along the
-// channel axis.  Shared layout: row k1 of a line at k1 (L2 + 1) (position
-// p = n1 L2 + n2 at p + p / L2), lines LP apart with LP = 16 / H mod 16 for
+// channel axis.  Shared layout: row k1 of a line at k1 RP, RP = L2 or L2 + 1,
+// whichever is odd (position p = n1 L2 + n2 at n1 RP + n2), lines LP apart with LP = 16 / H mod 16 for
 // H lines per half-warp (odd for H = 16): a half-warp's 64-bit accesses then
 // fall on distinct banks in both phases.
 //
@@ -71,7 +71,7 @@ __host__ __device__ constexpr bool fft2_half_applies() {
     return (KIND == PASS_FWD_FIRST || KIND == PASS_FWD_MID) ? L1 % 4 == 0 : L2 % 4 == 0;
 }
 
-__host__ __device__ constexpr int fft2_regs(int L2) { return L2 == 32 ? 80 : (L2 >= 20 ? 72 : 64); }
+__host__ __device__ constexpr int fft2_regs(int L2) { return L2 >= 25 ? 80 : (L2 >= 20 ? 72 : 64); }
 
 template <int L1, int L2, PassKind KIND, bool HALF>
 __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
@@ -87,7 +87,7 @@ __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
     constexpr bool FH = HALF && DIR < 0 && fft2_half_applies<L1, L2, KIND>();   // forward: n1 kept iff
     constexpr bool IH = HALF && DIR > 0 && fft2_half_applies<L1, L2, KIND>();   // inverse: k2 kept iff
     constexpr int Q = L / 4;
-    constexpr int RP = L2 + 1;   // row pitch inside a line
+    constexpr int RP = L2 | 1;   // row pitch inside a line (odd: no conflicts down a column)
     const int LP = a.TLP;        // line pitch (>= L1 RP, >= n_out)
     extern __shared__ float2 buf[];   // [TL][LP]
     const int lgTS = a.lgTS, lgTL = a.lgTL;
@@ -135,7 +135,7 @@ __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
                 }
             }
             float2* dst = buf + ln * LP;
-            for (int p = h + lane; p < L - h; p += 32) dst[p + p / L2] = make_float2(0.f, 0.f);
+            for (int p = h + lane; p < L - h; p += 32) dst[p + (RP - L2) * (p / L2)] = make_float2(0.f, 0.f);
             // image element e sits at position (e - n_in/2) mod L.  A row is loaded in
             // batches of NB elements per lane, one batch for rows of up to 384 elements at
             // sigma = 1.25; indices are clamped so the loads are unconditional and
@@ -145,7 +145,7 @@ __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
             if (!ok) {
                 for (int e = lane; e < n; e += 32) {
                     const int p = e < h ? e - h + L : e - h;
-                    dst[p + p / L2] = make_float2(0.f, 0.f);
+                    dst[p + (RP - L2) * (p / L2)] = make_float2(0.f, 0.f);
                 }
                 continue;
             }
@@ -172,7 +172,7 @@ __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
                         float sc = rs * dv[q];
                         sc *= kind == Dm1 ? (float)(e - nlast / 2) : wgt;
                         const int p = e < h ? e - h + L : e - h;
-                        dst[p + p / L2] = cscale(xv[q], sc);
+                        dst[p + (RP - L2) * (p / L2)] = cscale(xv[q], sc);
                     }
                 }
             }
@@ -373,8 +373,8 @@ __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
 
 namespace nj {
 
-// Launches k_line_fft2<L1, L2, KIND> when (L1, L2) has a compiled kernel.
-template <PassKind KIND>
+// Launches k_line_fft2<L1, L2, KIND> when (L1, L2) has a compiled kernel in the list.
+template <PassKind KIND, int LIST>
 cudaError_t launch_fft2_kind(int L1, int L2, const LinePass& a, dim3 grid, int threads, size_t smem, cudaStream_t s) {
 #define NJ_FFT2_CASE(A, B)                                                                   \
     if (L1 == A && L2 == B) {                                                                 \
@@ -389,7 +389,11 @@ cudaError_t launch_fft2_kind(int L1, int L2, const LinePass& a, dim3 grid, int t
         (void)launch_pdl(k_line_fft2<A, B, KIND, false>, grid, threads, smem, s, a);          \
         return cudaGetLastError();                                                            \
     }
-    NJ_FFT2_SIZES(NJ_FFT2_CASE)
+    if constexpr (LIST == 0) {
+        NJ_FFT2_SIZES_0(NJ_FFT2_CASE)
+    } else {
+        NJ_FFT2_SIZES_1(NJ_FFT2_CASE)
+    }
 #undef NJ_FFT2_CASE
     return cudaErrorInvalidValue;
 }

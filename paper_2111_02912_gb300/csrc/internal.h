@@ -274,22 +274,31 @@ __device__ __forceinline__ void line_tile(int64_t ntiles_s, uint32_t& tile_b, ui
 cudaError_t launch_line_pass(PassKind kind, const LinePass& a, dim3 grid, int threads, size_t smem,
                              cudaStream_t s);
 // Register-resident two-phase passes (k_line_fft2): factorisations L = L1 L2
-// with a compiled kernel, X(L1, L2), L1 <= L2 <= 32.  Launch with TL lines per
-// block (power of two, TL L2 threads, a multiple of 32, at most 512) and
-// TL (L + 1) complex of dynamic shared memory.
-#define NJ_FFT2_SIZES(X) \
+// with a compiled kernel, X(L1, L2), L1 even, L1 <= L2 <= 32, in two lists (compiled apart).  Launch
+// with TL lines per block (power of two, at least TL L2 threads, a multiple of 32, at most 512) and
+// TL LP complex of dynamic shared memory.  The second list holds the other grid edges of usual image
+// sides (60 .. 288 at sigma = 2): a factor that is a multiple of four (L1 forward, L2 inverse) also
+// prunes the zero half at compile time.
+#define NJ_FFT2_SIZES_0(X) \
     X(8, 8) X(8, 10) X(8, 12) X(8, 16) X(10, 16) X(12, 16) X(12, 20) X(16, 16) \
     X(16, 20) X(16, 24) X(20, 20) X(20, 24) X(16, 32) X(20, 32) X(24, 32) X(32, 32)
-template <PassKind KIND>
+#define NJ_FFT2_SIZES_1(X) \
+    X(10, 12) X(12, 12) X(12, 15) X(10, 20) X(12, 18) X(12, 24) X(12, 25) X(18, 20) \
+    X(18, 24) X(18, 25) X(24, 24)
+template <PassKind KIND, int LIST>
 cudaError_t launch_fft2_kind(int L1, int L2, const LinePass& a, dim3 grid, int threads, size_t smem, cudaStream_t s);
-inline bool fft2_factor(int L, int& L1, int& L2) {
+// The factors of L and the list they are in; false when L has no compiled kernel.
+inline bool fft2_factor(int L, int& L1, int& L2, int* list = nullptr) {
 #define NJ_FFT2_MATCH(A, B) \
     if (L == (A) * (B)) {   \
         L1 = A;             \
         L2 = B;             \
         return true;        \
     }
-    NJ_FFT2_SIZES(NJ_FFT2_MATCH)
+    if (list) *list = 0;
+    NJ_FFT2_SIZES_0(NJ_FFT2_MATCH)
+    if (list) *list = 1;
+    NJ_FFT2_SIZES_1(NJ_FFT2_MATCH)
 #undef NJ_FFT2_MATCH
     return false;
 }

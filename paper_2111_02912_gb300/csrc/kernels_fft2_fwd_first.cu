@@ -1,7 +1,7 @@
-// Register-resident two-phase line FFT, pass kind PASS_FWD_FIRST (one translation
-// unit per pass kind so that the kernels compile in parallel).
+// Register-resident two-phase line FFT, pass kind PASS_FWD_FIRST, list 0 of the line lengths (one
+// translation unit per pass kind and list so that the kernels compile in parallel).
 #include "fft_twostep.cuh"
 
 namespace nj {
-template cudaError_t launch_fft2_kind<PASS_FWD_FIRST>(int, int, const LinePass&, dim3, int, size_t, cudaStream_t);
+template cudaError_t launch_fft2_kind<PASS_FWD_FIRST, 0>(int, int, const LinePass&, dim3, int, size_t, cudaStream_t);
 }  // namespace nj

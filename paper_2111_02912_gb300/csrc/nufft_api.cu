@@ -726,14 +726,15 @@ int sort_join(nufft_plan_s* p, cudaStream_t s) {
     return NUFFT_OK;
 }
 
-// Two-phase line pass of kind `kind` (kernels instantiated one kind per translation unit).
-cudaError_t launch_line_pass2(PassKind kind, int L1, int L2, const LinePass& a, dim3 grid, int threads,
-                                     size_t smem, cudaStream_t s) {
+// Two-phase line pass of kind `kind` (kernels instantiated one kind and list of lengths per translation unit).
+template <int LIST>
+cudaError_t launch_line_pass2(PassKind kind, int L1, int L2, const LinePass& a, dim3 grid, int threads, size_t smem,
+                              cudaStream_t s) {
     switch (kind) {
-        case PASS_FWD_FIRST: return launch_fft2_kind<PASS_FWD_FIRST>(L1, L2, a, grid, threads, smem, s);
-        case PASS_FWD_MID: return launch_fft2_kind<PASS_FWD_MID>(L1, L2, a, grid, threads, smem, s);
-        case PASS_INV_MID: return launch_fft2_kind<PASS_INV_MID>(L1, L2, a, grid, threads, smem, s);
-        default: return launch_fft2_kind<PASS_INV_LAST>(L1, L2, a, grid, threads, smem, s);
+        case PASS_FWD_FIRST: return launch_fft2_kind<PASS_FWD_FIRST, LIST>(L1, L2, a, grid, threads, smem, s);
+        case PASS_FWD_MID: return launch_fft2_kind<PASS_FWD_MID, LIST>(L1, L2, a, grid, threads, smem, s);
+        case PASS_INV_MID: return launch_fft2_kind<PASS_INV_MID, LIST>(L1, L2, a, grid, threads, smem, s);
+        default: return launch_fft2_kind<PASS_INV_LAST, LIST>(L1, L2, a, grid, threads, smem, s);
     }
 }
 
@@ -744,11 +745,18 @@ struct Tile {
     int TB, TS, TL, threads;
     size_t smem;
     int L1, L2, LP;   // two-phase kernel: factors and shared line pitch
+    int list;         // ... and the list of lengths it is compiled in
 };
+
+cudaError_t launch_pass(PassKind kind, const Tile& t, const LinePass& a, dim3 grid, cudaStream_t s) {
+    if (!t.L1) return launch_line_pass(kind, a, grid, t.threads, t.smem, s);
+    return t.list ? launch_line_pass2<1>(kind, t.L1, t.L2, a, grid, t.threads, t.smem, s)
+                  : launch_line_pass2<0>(kind, t.L1, t.L2, a, grid, t.threads, t.smem, s);
+}
 
 Tile pick_tile(int L, int64_t B, int64_t S, PassKind kind, bool coil_sum, int n_out, bool pair = false) {
     Tile t{};
-    if (fft2_factor(L, t.L1, t.L2)) {
+    if (fft2_factor(L, t.L1, t.L2, &t.list)) {
         // 8 adjacent lines (64-byte segments along the channel axis), two or three blocks per SM:
         // measured faster than 4 or 16 lines on the 640-point passes.  The coil-summing last
         // inverse pass takes 8 coils per block when its two coil chunks add into a cleared image
@@ -761,14 +769,14 @@ Tile pick_tile(int L, int64_t B, int64_t S, PassKind kind, bool coil_sum, int n_
         t.TS = std::min<int>(TL, pow2_ceil(S));
         t.TB = std::min<int>(TL / t.TS, pow2_ceil(B));
         t.TL = t.TB * t.TS;
-        while ((t.TL * t.L2) % 32 != 0) {   // whole warps; extra lines are masked
+        while (t.L2 <= 12 && (t.TL * t.L2) % 32 != 0) {   // whole warps; extra lines are masked
             t.TB *= 2;
             t.TL *= 2;
         }
-        t.threads = t.TL * t.L2;
-        // line pitch: >= L1 (L2 + 1), congruent to 16 / H mod 16 for H lines per half-warp
-        const int H = std::min(t.TL, 16), want = H == 16 ? 1 : 16 / H;
-        t.LP = t.L1 * (t.L2 + 1);
+        t.threads = (t.TL * t.L2 + 31) / 32 * 32;   // ... or extra threads
+        // line pitch: >= L1 (L2 | 1), congruent to 16 / H mod 16 for H lines per half-warp
+        const int H = std::min(t.TL, 16), want = (H == 16 ? 1 : 16 / H) % 16;
+        t.LP = t.L1 * (t.L2 | 1);
         while (t.LP % 16 != want) ++t.LP;
         t.smem = (size_t)t.TL * t.LP * sizeof(float2);
         return t;
@@ -839,10 +847,7 @@ int forward_grids(nufft_plan_s* p, int C, int nd, int has_plain, const float2* x
         a.magic_n = magic_of((uint32_t)a.n_out);
         a.ntiles_s = (S + t.TS - 1) / t.TS;
         const dim3 grid = line_grid((B + t.TB - 1) / t.TB, a.ntiles_s);
-        int st = launch(p, k == 0 ? PK_FFT_FWD_FIRST : PK_FFT_FWD_MID, s, [&] {
-            return t.L1 ? launch_line_pass2(kind, t.L1, t.L2, a, grid, t.threads, t.smem, s)
-                        : launch_line_pass(kind, a, grid, t.threads, t.smem, s);
-        });
+        int st = launch(p, k == 0 ? PK_FFT_FWD_FIRST : PK_FFT_FWD_MID, s, [&] { return launch_pass(kind, t, a, grid, s); });
         if (st) return st;
         in = out;
     }
@@ -999,10 +1004,7 @@ int inverse_passes(nufft_plan_s* p, int C, const float2* smaps, float2* xout, cu
         a.magic_n = magic_of((uint32_t)a.n_out);
         a.ntiles_s = chunks;
         const dim3 grid = line_grid((B + t.TB - 1) / t.TB, chunks);
-        st = launch(p, last ? PK_FFT_INV_LAST : PK_FFT_INV_MID, s, [&] {
-            return t.L1 ? launch_line_pass2(kind, t.L1, t.L2, a, grid, t.threads, t.smem, s)
-                        : launch_line_pass(kind, a, grid, t.threads, t.smem, s);
-        });
+        st = launch(p, last ? PK_FFT_INV_LAST : PK_FFT_INV_MID, s, [&] { return launch_pass(kind, t, a, grid, s); });
         if (st) return st;
         if (part) {
             st = launch(p, PK_SUM_CHUNKS, s, [&] { return launch_sum_chunks(part, chunks, p->Nimg, xout, s); });
