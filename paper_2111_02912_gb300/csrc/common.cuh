@@ -152,9 +152,11 @@ inline cudaError_t launch_pdl_cluster(void (*kernel)(Params...), unsigned blocks
 
 // Every thread of the cluster waits for all of them; what they wrote to global memory before is seen
 // by (L2) loads after.  The hardware schedules a cluster's blocks together, so this always ends.
+// Each thread arrives by itself: the .aligned form asks that a whole warp executes it together, which
+// nothing ensures after loops whose trip counts differ between the threads.
 __device__ __forceinline__ void cluster_barrier() {
     __threadfence();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" "barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    asm volatile("barrier.cluster.arrive.release;\n" "barrier.cluster.wait.acquire;\n" ::: "memory");
 }
 
 }  // namespace nj

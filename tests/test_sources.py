@@ -39,3 +39,14 @@ def test_no_kernel_is_launched_without_launch_pdl():
     for name, text in _sources():
         code = _strip_comments(text)
         assert "<<<" not in code, "%s launches a kernel with <<< >>> instead of launch_pdl" % name
+
+
+def test_cluster_barriers_do_not_ask_for_a_converged_warp():
+    """barrier.cluster with .aligned is undefined when the threads of a warp do not execute it together,
+    and the cluster kernels reach it behind loops that the threads leave at different times."""
+    found = 0
+    for name, text in _sources():
+        for m in re.finditer(r"barrier\.cluster\.(?:arrive|wait)[.\w]*", _strip_comments(text)):
+            found += 1
+            assert "aligned" not in m.group(0), "%s: %s" % (name, m.group(0))
+    assert found >= 2
