@@ -130,7 +130,9 @@ int nufft_plan(nufft_plan_t* out, const nufft_opts* o, int64_t m, const float* o
  * they are fixed: the bin sort computes each point's window start and its D*J
  * kernel weights once, and every later gather and spread of these points reads
  * them.  m may differ from the plan's current m; growing past the capacity
- * reallocates (synchronising).  The call copies omega into the plan on `stream`
+ * reallocates (synchronising); when that fails (NUFFT_ERR_OOM) the plan is left
+ * without points and refuses every call with the same status until an
+ * nufft_set_points succeeds.  The call copies omega into the plan on `stream`
  * (the caller's buffer is free once that copy has run); the bin sort itself runs
  * in the next call that needs the points, on the plan's own stream, beside that
  * call's FFT passes. */

@@ -78,6 +78,7 @@ struct nufft_plan_s {
     double sigma = 2.0, beta = 0.0;
     int maxC = 1;
     int64_t M = 0, M_cap = 0;
+    bool no_points = false;   // the point storage could not be allocated
     int64_t Nimg = 1, Ktot = 1;
     KbPoly kb{};
     float* d_deap[3] = {nullptr, nullptr, nullptr};
@@ -445,19 +446,20 @@ size_t point_bytes(const nufft_plan_s& p, int64_t cap) {
     return b;
 }
 
-int alloc_points(nufft_plan_s* p, int64_t cap) {
-    cudaFree(p->d_items); cudaFree(p->d_local); cudaFree(p->d_keyid); cudaFree(p->d_pidx); cudaFree(p->d_pfrac);
-    cudaFree(p->d_pw); cudaFree(p->d_om); cudaFree(p->d_ys); cudaFree(p->d_hits); cudaFree(p->d_hits_tmp);
-    p->d_items = nullptr; p->d_local = p->d_keyid = nullptr; p->d_pidx = nullptr; p->d_pfrac = nullptr;
-    p->d_pw = nullptr;
-    p->d_om = nullptr;
-    p->d_ys = nullptr;
-    p->d_hits = nullptr;
-    p->d_hits_tmp = nullptr;
-    cudaFree(p->d_partial); cudaFree(p->d_counters); cudaFree(p->d_splits);
-    p->d_partial = nullptr;
-    p->d_counters = nullptr;
-    p->d_splits = nullptr;
+void free_points(nufft_plan_s* p) {
+    auto drop = [](auto*& q) {
+        cudaFree(q);
+        q = nullptr;
+    };
+    drop(p->d_items); drop(p->d_local); drop(p->d_keyid); drop(p->d_pidx); drop(p->d_pfrac); drop(p->d_pw);
+    drop(p->d_om); drop(p->d_ys); drop(p->d_hits); drop(p->d_hits_tmp); drop(p->d_partial); drop(p->d_counters);
+    drop(p->d_splits);
+    p->M = p->M_cap = 0;
+    p->sort_pending = p->cap_pending = false;
+    p->no_points = true;
+}
+
+int alloc_point_arrays(nufft_plan_s* p, int64_t cap) {
     const size_t c = (size_t)std::max<int64_t>(cap, 1);
     if (p->strip) {
         p->hit_cap = (int64_t)c * strip_hits_per_point(*p);
@@ -489,7 +491,26 @@ int alloc_points(nufft_plan_s* p, int64_t cap) {
         cudaGetLastError();
         return fail(NUFFT_ERR_OOM, "device allocation of point arrays failed");
     }
+    return NUFFT_OK;
+}
+
+// New storage for cap points in place of the old.  When it fails the plan has none: what was allocated
+// is given back, and its calls are refused (check_points) until a set_points succeeds.
+int alloc_points(nufft_plan_s* p, int64_t cap) {
+    free_points(p);
+    const int st = alloc_point_arrays(p, cap);
+    if (st) {
+        free_points(p);
+        return st;
+    }
     p->M_cap = cap;
+    p->no_points = false;
+    return NUFFT_OK;
+}
+
+int check_points(const nufft_plan_s* p) {
+    if (p->no_points)
+        return fail(NUFFT_ERR_OOM, "the plan has no point storage: its last nufft_set_points ran out of device memory");
     return NUFFT_OK;
 }
 
@@ -594,10 +615,10 @@ bool capture_id(cudaStream_t s, unsigned long long& id) {
 int do_set_points(nufft_plan_s* p, int64_t m, const float* omega, cudaStream_t s) {
     if (m < 0 || m > (int64_t)INT32_MAX) return fail(NUFFT_ERR_INVALID_ARG, "m out of range");
     if (m > 0 && !omega) return fail(NUFFT_ERR_INVALID_ARG, "omega is NULL");
-    if (m > p->M_cap) {
+    if (m > p->M_cap || p->no_points) {
         NJ_CUDA(cudaStreamSynchronize(s));
         if (p->aux) NJ_CUDA(cudaStreamSynchronize(p->aux));
-        int st = alloc_points(p, m);
+        int st = alloc_points(p, std::max<int64_t>(m, 1));
         if (st) return st;
         p->bytes = 0;
     }
@@ -1063,7 +1084,7 @@ int gather_cpl(const GatherArgs& g) {
 int check_call(nufft_plan_s* p, int C) {
     if (!p) return fail(NUFFT_ERR_INVALID_ARG, "plan is NULL");
     if (C < 1 || C > p->maxC) return fail(NUFFT_ERR_INVALID_ARG, "C must lie in [1, max_coils]");
-    return NUFFT_OK;
+    return check_points(p);
 }
 
 }  // namespace
@@ -1193,6 +1214,8 @@ int nufft_set_points(nufft_plan_t p, int64_t m, const float* omega, void* stream
 
 int nufft_sort_points(nufft_plan_t p, void* stream) {
     if (!p) return fail(NUFFT_ERR_INVALID_ARG, "plan is NULL");
+    int st;
+    if ((st = check_points(p))) return st;
     cudaStream_t s = (cudaStream_t)stream;
     p->last_stream = s;
     return finish_call(p, s, sort_rest(p, s));
