@@ -176,7 +176,8 @@ int nufft_vjp_omega_x(nufft_plan_t p, int C, const nufft_cfloat* x, const nufft_
  * overlap.  `work` is nufft_cg_work_bytes bytes of device memory, 16-byte aligned, used until the
  * work queued on `stream` has finished.  The whole solve is queued without waiting for the device:
  * the scalars stay there, and the k-space values go from the gather to the spread in the sorted
- * order, without passing through the caller's. */
+ * order, without passing through the caller's.  Once the residual is zero, further steps leave x as
+ * it is. */
 size_t nufft_cg_work_bytes(nufft_plan_t p, int C, int has_maps);
 int nufft_cg_normal(nufft_plan_t p, int C, const nufft_cfloat* b, const nufft_cfloat* smaps, float lam, int iters,
                     nufft_cfloat* x, void* work, size_t work_bytes, void* stream);

@@ -5,13 +5,14 @@
 //   k_cg_update  alpha = <r,r> / <p, F p>;  x += alpha p;  r -= alpha (q + lam p);  partial sums of <r,r>
 //   k_cg_dir     p = r + (<r,r>_new / <r,r>_old) p
 // The scalars stay on the device: every block adds the partial sums of the kernel before it by
-// itself, in block order, so that a solve never waits for the host and repeats bit by bit.  The
-// vectors are read and written once per step (7 reads, 3 writes an iteration), which is all these
+// itself, in block order, so that a solve never waits for the host and, on a deterministic plan, repeats
+// bit by bit.  The vectors are read and written once per step (7 reads, 3 writes an iteration), which is all these
 // kernels do; they are launch-bound up to a few hundred thousand elements.  The same algebra as
 // about twenty tensor operations per iteration kept the host busy for 340 us beside 115 us of
 // normal product (320^2, 16 coils); a solve of 10 iterations and its gradient went from 6732 to
-// 2957 us, with an error against FP64 of 5.4e-7 instead of 9.5e-7.  Sums run in FP32 within
-// a thread (a few dozen terms at most) and in FP64 across threads and blocks.
+// 2957 us, with errors against FP64 of 6e-7 to 7e-7 (6e-7 to 1.6e-6 before).  Products and sums of the
+// scalars are FP64: the square of any FP32 number is then above zero, so <r,r> is zero only where r is,
+// and the iteration then stays where it is (alpha = beta = 0) instead of dividing zero by zero.
 #include <algorithm>
 
 #include "internal.h"
@@ -41,37 +42,44 @@ __device__ __forceinline__ double cg_total(const double* part, int nb) {
     return cg_block_sum(v);
 }
 
+// s + |v|^2 and s + Re{conj(a) b}, exact products.
+__device__ __forceinline__ double cg_add_sqr(double s, float2 v) {
+    return fma((double)v.x, (double)v.x, fma((double)v.y, (double)v.y, s));
+}
+__device__ __forceinline__ double cg_add_dot(double s, float2 a, float2 b) {
+    return fma((double)a.x, (double)b.x, fma((double)a.y, (double)b.y, s));
+}
+
 __global__ void __launch_bounds__(kCgThreads) k_cg_start(CgArgs a) {
     pdl_wait();
-    float s = 0.f;
+    double s = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * kCgThreads + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * kCgThreads) {
         const float2 b = a.b[i];
         a.x[i] = make_float2(0.f, 0.f);
         a.r[i] = b;
         a.p[i] = b;
-        s = fmaf(b.x, b.x, fmaf(b.y, b.y, s));
+        s = cg_add_sqr(s, b);
     }
-    const double t = cg_block_sum((double)s);
+    const double t = cg_block_sum(s);
     if (threadIdx.x == 0) a.rr[blockIdx.x] = t;
 }
 
 __global__ void __launch_bounds__(kCgThreads) k_cg_dot(CgArgs a) {
     pdl_wait();
-    float s = 0.f;
+    double s = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * kCgThreads + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * kCgThreads) {
         const float2 p = a.p[i], q = a.q[i];
-        const float fx = fmaf(a.lam, p.x, q.x), fy = fmaf(a.lam, p.y, q.y);
-        s = fmaf(p.x, fx, fmaf(p.y, fy, s));
+        s = cg_add_dot(s, p, make_float2(fmaf(a.lam, p.x, q.x), fmaf(a.lam, p.y, q.y)));
     }
-    const double t = cg_block_sum((double)s);
+    const double t = cg_block_sum(s);
     if (threadIdx.x == 0) a.pq[blockIdx.x] = t;
 }
 
 __global__ void __launch_bounds__(kCgThreads) k_cg_update(CgArgs a) {
     pdl_wait();
     const double rr = cg_total(a.rr, gridDim.x), pq = cg_total(a.pq, gridDim.x);
-    const float alpha = (float)(rr / pq);
-    float s = 0.f;
+    const float alpha = pq == 0.0 ? 0.f : (float)(rr / pq);   // p = 0 (or F p = 0): no step left
+    double s = 0.0;
     for (int64_t i = (int64_t)blockIdx.x * kCgThreads + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * kCgThreads) {
         const float2 p = a.p[i], q = a.q[i];
         float2 x = a.x[i], r = a.r[i];
@@ -81,16 +89,16 @@ __global__ void __launch_bounds__(kCgThreads) k_cg_update(CgArgs a) {
         r.y = fmaf(-alpha, fmaf(a.lam, p.y, q.y), r.y);
         a.x[i] = x;
         a.r[i] = r;
-        s = fmaf(r.x, r.x, fmaf(r.y, r.y, s));
+        s = cg_add_sqr(s, r);
     }
-    const double t = cg_block_sum((double)s);
+    const double t = cg_block_sum(s);
     if (threadIdx.x == 0) a.rr_new[blockIdx.x] = t;
 }
 
 __global__ void __launch_bounds__(kCgThreads) k_cg_dir(CgArgs a) {
     pdl_wait();
     const double rn = cg_total(a.rr_new, gridDim.x), rr = cg_total(a.rr, gridDim.x);
-    const float beta = (float)(rn / rr);
+    const float beta = rr == 0.0 ? 0.f : (float)(rn / rr);
     for (int64_t i = (int64_t)blockIdx.x * kCgThreads + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * kCgThreads) {
         const float2 r = a.r[i], p = a.p[i];
         a.p[i] = make_float2(fmaf(beta, p.x, r.x), fmaf(beta, p.y, r.y));
