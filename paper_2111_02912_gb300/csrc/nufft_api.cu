@@ -527,7 +527,9 @@ StripTables strip_tables(const nufft_plan_s& p) {
     t.splits = p.d_splits;
     t.nitems = p.d_nitems;
     t.P = p.strip_P;
-    t.slots = p.strip_slots;
+    // by the points of this sort, not by the storage (strip_slots, never fewer): the cut into parts, and with it
+    // the order of the sums, must not depend on how many points the plan has held before
+    t.slots = strip_slots_for(p, std::max<int64_t>(p.M, 1));
     return t;
 }
 
@@ -892,7 +894,7 @@ int adjoint_impl(nufft_plan_s* p, int C, const float2* y, const float2* smaps, f
         ta.pts = PointsView{p->d_pidx, p->d_pfrac, p->M, p->d_pw, p->ws, p->wd};
         ta.g = strip_geom(*p);
         ta.t = strip_tables(*p);
-        ta.max_items = p->nunits + p->strip_slots;
+        ta.max_items = p->nunits + ta.t.slots;
         ta.C = C;
         const int cpt = 64 / p->NSL;   // coils per warp
         ta.ncg = (C + cpt - 1) / cpt;
