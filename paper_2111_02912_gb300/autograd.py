@@ -135,19 +135,29 @@ def cg_solve(apply_F, b, iters, x0=None):
     return x
 
 
+_OWN = (NufftOperator.forward, NufftOperator.adjoint, Plan.forward, Plan.adjoint)
+
+
+def _applies_own_methods(op):
+    """Whether op.forward and op.adjoint are the ones above on a plan with its own: not a subclass's, and not
+    replaced on the operator, its class, the plan or the plan's class."""
+    if type(op) is not NufftOperator or type(op.plan) is not Plan:
+        return False
+    calls = (op.forward, op.adjoint, op.plan.forward, op.plan.adjoint)
+    return all(getattr(c, "__func__", None) is f and c.__self__ is o
+               for c, f, o in zip(calls, _OWN, (op, op, op.plan, op.plan)))
+
+
 def _solve_normal(op, b, lam, iters):
     """iters CG steps on (E'E + lam I) x = b: the library's solver where it applies, else cg_solve.
 
-    The solver takes the operator as it is (its own E and E', not a subclass's or a replaced method)
-    and b shaped like the adjoint's output.  One step of the vector algebra is three launches there
+    The solver applies the plan's own E and E', so it takes operators that would call just these, and b
+    shaped like the adjoint's output.  One step of the vector algebra is three launches there
     and about twenty small ones here, which held the GPU up: psd_inverse and its gradient at 320^2,
     16 coils, 51,200 points, ten iterations each way: 6732 -> 2957 us.
     """
-    one = op.smaps is not None if isinstance(op, NufftOperator) else False
-    plain = (type(op) is NufftOperator and type(op.plan) is Plan and b.is_cuda and b.dtype == torch.complex64
-             and not {"forward", "adjoint"} & op.__dict__.keys() and isinstance(lam, (int, float)) and iters > 0
-             and tuple(b.shape if one else b.shape[1:]) == op.shape)
-    if plain:
+    if (_applies_own_methods(op) and b.is_cuda and b.dtype == torch.complex64 and isinstance(lam, (int, float))
+            and iters > 0 and tuple(b.shape if op.smaps is not None else b.shape[1:]) == op.shape):
         return op.plan.cg_normal(b.resolve_conj().contiguous(), lam, iters, op.smaps)
     return cg_solve(lambda v: op.adjoint(op.forward(v)) + lam * v, b, iters)
 
