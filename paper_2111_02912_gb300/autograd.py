@@ -158,7 +158,7 @@ def _solve_normal(op, b, lam, iters):
     """
     if (_applies_own_methods(op) and b.is_cuda and b.dtype == torch.complex64 and isinstance(lam, (int, float))
             and iters > 0 and tuple(b.shape if op.smaps is not None else b.shape[1:]) == op.shape):
-        return op.plan.cg_normal(b.resolve_conj().contiguous(), lam, iters, op.smaps)
+        return op.plan.cg_normal(b.resolve_conj().resolve_neg().contiguous(), lam, iters, op.smaps)
     return cg_solve(lambda v: op.adjoint(op.forward(v)) + lam * v, b, iters)
 
 

@@ -1,5 +1,5 @@
 """psd_inverse solves with the operator that it is given: replaced methods, of the object, its class or its
-plan, are what the iteration applies."""
+plan, are what the iteration applies, and b's values count, not its storage."""
 import pytest
 
 from gpu_helpers import host, make_case, rel, to_dev
@@ -32,3 +32,12 @@ def test_replaced_methods_are_applied(where, monkeypatch):
             monkeypatch.setattr(target, name, lambda *a, plain=plain, **k: 2.0 * plain(*a, **k))
     want = cg_solve(lambda v: op.adjoint(op.forward(v)) + LAM * v, b, ITERS)
     assert rel(host(psd_inverse(b, om, op, LAM, ITERS)), host(want)) < TOL
+
+
+def test_values_of_a_negative_view():
+    import torch
+
+    from paper_2111_02912_gb300.autograd import psd_inverse
+    om, b, op = _operator(96)
+    got, want = psd_inverse(torch._neg_view(b), om, op, LAM, ITERS), psd_inverse(b, om, op, LAM, ITERS)
+    assert rel(host(got), -host(want)) < TOL
