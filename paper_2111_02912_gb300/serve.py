@@ -173,7 +173,7 @@ class Server:
         S = req.smaps
         if req.kind == "recon":
             b = plan.adjoint(req.y, S)
-            req.result = plan.cg_normal(b, req.lam, req.iters, S)
+            req.result = plan.cg_normal(b, req.lam, max(req.iters, 0), S)
         else:   # traj_grad: L = ||E x - y||^2, v = 2 (E x - y)
             v = 2.0 * (plan.forward(req.x, S) - req.y)
             go, _ = plan.vjp_omega_x(req.x, v, S, need_omega=True, need_x=False)
