@@ -599,10 +599,16 @@ SortArgs sort_args(nufft_plan_s* p, const float* omega) {
 
 int sort_rest(nufft_plan_s* p, cudaStream_t s);
 
-// The one-launch sort runs up to this many points (one per thread of its cluster), and bins and strip
-// units (which one block scans).
+// The one-launch sort saves the host five launches, about 7 us, and makes the device wait longer (one block scans
+// the bins and plans the strip units, and the first gather waits for the hit lists too).  It is taken where the
+// host bounds a step: eager calls on 2-D plans of up to 4096 points (one per thread of its cluster), 1280 strip
+// units and 1024 bins.  Eager set_points + forward + VJP, separate launches -> one, 80 .. 4096 points: 40^2,
+// 8 coils 67 -> 53..61 us, 128^2, 16 coils (1024 units) 68 -> 56..67, 192^2, 8 coils (1152) 66 -> 52..63; beyond,
+// 256^2, 8 coils (2048) 66..71 -> 70..78, 320^2, 1 coil (1600 bins) 68 -> 60..70, 384^2, 16 coils 199 -> 226,
+// and 3-D 40^3, 1 coil 140 -> 160.  Replayed from a graph, where launches cost the host nothing, the separate
+// ones take 0.78 .. 1.0 of its time: recorded sorts never use it.
 constexpr int64_t kSmallSortPoints = 4096;
-constexpr int kSmallSortTables = 16384;
+constexpr int kSmallSortUnits = 1280, kSmallSortBins = 1024;
 
 // True, with the capture sequence id, when s is recording into a CUDA graph.
 bool capture_id(cudaStream_t s, unsigned long long& id) {
@@ -665,11 +671,11 @@ int sort_rest(nufft_plan_s* p, cudaStream_t s) {
         ss = p->aux;
     }
     int st;
-    if (p->strip && !p->deterministic && p->M > 0 && p->M <= kSmallSortPoints && p->nbins <= kSmallSortTables &&
-        p->nunits <= kSmallSortTables) {
-        const bool clear = capturing || !p->kcount_clear;
+    if (p->strip && p->D == 2 && !p->deterministic && !capturing && p->M > 0 && p->M <= kSmallSortPoints &&
+        p->nbins <= kSmallSortBins && p->nunits <= kSmallSortUnits) {
+        const bool clear = !p->kcount_clear;
         if ((st = launch(p, PK_SORT_SMALL, ss, [&] { return launch_sort_small(a, clear, ss); }))) return st;
-        if (!capturing) p->kcount_clear = true;
+        p->kcount_clear = true;
         if (p->aux) {   // records and strip tables are ready together
             NJ_CUDA(cudaEventRecord(p->join_ev, p->aux));
             p->join_pending = true;
