@@ -552,8 +552,11 @@ StripGeom strip_geom(const nufft_plan_s& p) {
 
 // From this many points the hits of 2-D strips are collected per block too (kernels_strip.cu): 384^2, 32
 // coils, 200,000 points: scatter 34.5 -> 25.7 us, fill 35.2 -> 16.2, count 14.9, the step 806 -> 789; at 51,200
-// points the extra launch costs what it gains (191.3 -> 191.0).  3-D: always.
-constexpr int64_t kHashHitPoints = 100000;
+// points the extra launch costs what it gains (191.3 -> 191.0).  3-D: always.  From kHashHitCrowded points also
+// where the points crowd the units, 32 or more to each: one global atomic per hit then meets others on its counter
+// (set_points and adjoint of uniform points, per hit -> per block, 64^2, 16 coils, 30,000 points 129 -> 89 us,
+// 128^2, 4 coils, 60,000 153 -> 107, 256^2, 1 coil, 30,000 68 -> 63; at 5000 points 51 -> 54).
+constexpr int64_t kHashHitPoints = 100000, kHashHitCrowded = 16384;
 
 SortArgs sort_args(nufft_plan_s* p, const float* omega) {
     SortArgs a{};
@@ -590,7 +593,7 @@ SortArgs sort_args(nufft_plan_s* p, const float* omega) {
     a.tab_L = (float)p->tab_L;
     a.tab_n = p->tab_n;
     a.strip = p->strip ? 1 : 0;
-    a.hash_hits = p->strip && (p->D == 3 || p->M >= kHashHitPoints) ? 1 : 0;
+    a.hash_hits = p->strip && (p->D == 3 || p->M >= kHashHitPoints || (p->M >= kHashHitCrowded && p->M >= 32 * (int64_t)p->nunits)) ? 1 : 0;
     a.nunits = p->nunits;
     a.sg = strip_geom(*p);
     a.st = strip_tables(*p);
