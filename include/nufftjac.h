@@ -84,8 +84,9 @@ typedef struct {
                           calls) */
     int spread_variant; /* adjoint spread kernel: NUFFT_SPREAD_AUTO (0), _STRIPS, _TILES, _GENERAL */
     int strip_part;   /* strip spread: hits one warp adds before a unit is split into parts
-                         (a power of two, 8..4096; 0 -> 32); longer where the
-                         parts' sums would need too much memory */
+                         (a power of two, 8..4096; 0 -> 32, longer where a unit's
+                         parts would take long to add); longer where the parts'
+                         sums would need too much memory */
     int kernel_mode;  /* how the interpolation weights psi(u) are evaluated (once per omega, by the
                          bin sort): NUFFT_KERNEL_DIRECT (0), the Kaiser-Bessel function itself as
                          its I0 power series in FP32; NUFFT_KERNEL_TABLE, psi sampled at

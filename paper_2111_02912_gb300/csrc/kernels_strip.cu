@@ -104,13 +104,13 @@ __device__ __forceinline__ void block_scan_tiles(int n, int (&carry)[V], Get get
 // --------------------------------------------------------------- sort tables
 // The plan in two launches of 256-thread blocks (unit b * 256 + t in block b, thread t).  Split
 // parts are counted for P * 2^L, L = 0..11: the smallest level whose split parts fit the partial
-// slots is used.  (a) Per block and level: hits, split parts and whole units.  (b) Every block sums
+// slots (and, with the default P, are long enough for the heaviest unit) is used.  (a) Per block and level: hits, split parts and whole units.  (b) Every block sums
 // the totals of the blocks before it, picks the level, scans its own units and writes their hit
 // offsets and items (split parts first: they start in the first wave), clearing the hit counts
 // (the next sort's scatter counts into them) and the fill cursors.
 constexpr int kPlanThreads = 256;
-constexpr int kPlanVals = 1 + 2 * kPlanLevels;   // hits, then split parts and whole units per level
-
+constexpr int kPlanSums = 1 + 2 * kPlanLevels;   // hits, then split parts and whole units per level
+constexpr int kPlanVals = kPlanSums + 1;         // ... and the hits of the heaviest unit
 
 __global__ void __launch_bounds__(kPlanThreads) k_strip_plan_a(SortArgs a) {
     pdl_wait();
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_strip_plan_a(SortArgs a) {
     const int u = blockIdx.x * kPlanThreads + t;
     const int h = u < a.nunits ? T.hcount[u] : 0;
     const int lgP = 31 - __clz(T.P);
-    int v[kPlanVals];
+    int v[kPlanSums];
     v[0] = h;
 #pragma unroll
     for (int L = 0; L < kPlanLevels; ++L) {
@@ -129,16 +129,16 @@ __global__ void __launch_bounds__(kPlanThreads) k_strip_plan_a(SortArgs a) {
         v[2 + 2 * L] = u < a.nunits && parts == 1 ? 1 : 0;
     }
 #pragma unroll
-    for (int q = 0; q < kPlanVals; ++q) {
-        int x = v[q];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    for (int q = 0; q < kPlanSums; ++q) {
+        const int x = __reduce_add_sync(0xffffffffu, v[q]);
         if (lane == 0) sh[q][w] = x;
     }
+    const int hw = __reduce_max_sync(0xffffffffu, h);
+    if (lane == 0) sh[kPlanSums][w] = hw;
     __syncthreads();
     if (t < kPlanVals) {
         int x = 0;
-        for (int k = 0; k < kPlanThreads / 32; ++k) x += sh[t][k];
+        for (int k = 0; k < kPlanThreads / 32; ++k) x = t < kPlanSums ? x + sh[t][k] : max(x, sh[t][k]);
         T.partial_sums[blockIdx.x * kPlanVals + t] = x;
     }
 }
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_strip_plan_b(SortArgs a) {
         int tot = 0, pre = 0;
         for (int k = 0; k < nblk; ++k) {
             const int x = T.partial_sums[k * kPlanVals + t];
-            tot += x;
+            tot = t < kPlanSums ? tot + x : max(tot, x);
             if (k < b) pre += x;
         }
         s_tot[t] = tot;
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_strip_plan_b(SortArgs a) {
     }
     __syncthreads();
     int L = 0;
-    while (L < kPlanLevels - 1 && s_tot[1 + 2 * L] > T.slots) ++L;
+    while (L < kPlanLevels - 1 && (plan_too_short(T, s_tot[kPlanSums], L) || s_tot[1 + 2 * L] > T.slots)) ++L;
     const bool fits = s_tot[1 + 2 * L] <= T.slots;
     const int lgP = (31 - __clz(T.P)) + L;
     const int H = fits ? s_tot[1 + 2 * L] : 0;   // split parts (items of split units come first)

@@ -89,6 +89,7 @@ struct nufft_plan_s {
     bool cell_spread = false;   // spread by the row-owner tile kernel (else the general kernel)
     // strip spread (2-D and 3-D): strip units of NSL rows x kStripW columns of the last axis
     bool strip = false;
+    bool part_auto = true;         // strip_P is the default, not the caller's
     bool deterministic = false;    // stable bin order and hit lists ordered by sorted point
     int kernel_mode = NUFFT_KERNEL_DIRECT, tab_L = 0, tab_n = 0;   // table mode: L samples per unit
     int gather_variant = NUFFT_GATHER_AUTO;
@@ -330,6 +331,7 @@ int validate_opts(const nufft_opts* o, nufft_plan_s& p) {
             if (o->strip_part < 8 || o->strip_part > 4096 || (o->strip_part & (o->strip_part - 1)))
                 return fail(NUFFT_ERR_INVALID_ARG, "strip_part must be a power of two in [8, 4096]");
             p.strip_P = o->strip_part;
+            p.part_auto = false;
         }
         p.deterministic = o->deterministic != 0;
         if (p.deterministic && !p.strip)
@@ -527,6 +529,7 @@ StripTables strip_tables(const nufft_plan_s& p) {
     t.splits = p.d_splits;
     t.nitems = p.d_nitems;
     t.P = p.strip_P;
+    t.auto_part = p.part_auto ? 1 : 0;
     // by the points of this sort, not by the storage (strip_slots, never fewer): the cut into parts, and with it
     // the order of the sums, must not depend on how many points the plan has held before
     t.slots = strip_slots_for(p, std::max<int64_t>(p.M, 1));
