@@ -21,7 +21,7 @@
 // Pass kinds: FWD_FIRST takes its input from the image (scaling s_n of the
 // Appendix, coil map of Sec. II-G, coordinate weight r^[d] of Eq. (e,Ax), zero
 // padding) with loads coalesced along the image row, straight into phase 1 for
-// sigma = 2, else by way of shared memory; FWD_MID reads only the
+// sigma = 2 (but for 512 and 1024 points), else by way of shared memory; FWD_MID reads only the
 // n_in nonzero positions of its input lines; INV_MID keeps the n_out cropped
 // positions; INV_LAST crops, stages the line in shared memory, then applies
 // the scaling and conj(s_c) and sums the tile's coils with loads and stores
@@ -108,7 +108,9 @@ __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
     const float* deap_last = a.im.deap[Dm1];
 
     // ---------------------------------------------------------------- input
-    constexpr bool DIRECT = KIND == PASS_FWD_FIRST && FH;   // phase 1 reads the image itself
+    // Phase 1 reads the image itself; 512- and 1024-point lines go through shared memory, faster there from 16 channels
+    // on (256^2, 20 coils: 18.8 -> 17.0 us, 512^2, 32 coils: 75.5 -> 68.5; one channel 9.1 -> 10.0).
+    constexpr bool DIRECT = KIND == PASS_FWD_FIRST && FH && !(L2 == 32 && L1 % 16 == 0);
     if constexpr (KIND == PASS_FWD_FIRST && !DIRECT) {
         const int warp = tid >> 5, lane = tid & 31, nwarps = blockDim.x >> 5;
         // Lines are (image row, channel); channel = dblk * C + coil, dblk 0 the
@@ -135,12 +137,13 @@ __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
                 }
             }
             float2* dst = buf + ln * LP;
-            for (int p = h + lane; p < L - h; p += 32) dst[p + (RP - L2) * (p / L2)] = make_float2(0.f, 0.f);
+            if (!FH)   // zero padding (with FH the padded registers are never read)
+                for (int p = h + lane; p < L - h; p += 32) dst[p + (RP - L2) * (p / L2)] = make_float2(0.f, 0.f);
             // image element e sits at position (e - n_in/2) mod L.  A row is loaded in
-            // batches of NB elements per lane, one batch for rows of up to 384 elements at
-            // sigma = 1.25; indices are clamped so the loads are unconditional and
+            // batches of NB elements per lane, one batch for rows of up to 384 elements;
+            // indices are clamped so the loads are unconditional and
             // independent (all in flight before the first use).
-            constexpr int NB = (L * 4 / 5 + 31) / 32 < 12 ? (L * 4 / 5 + 31) / 32 : 12;
+            constexpr int NB1 = ((FH ? L / 2 : L * 4 / 5) + 31) / 32, NB = NB1 < 12 ? NB1 : 12;
             const int n = a.n_in;
             if (!ok) {
                 for (int e = lane; e < n; e += 32) {
@@ -220,7 +223,8 @@ __global__ void __maxnreg__(fft2_regs(L2)) k_line_fft2(LinePass a) {
         } else if constexpr (KIND == PASS_FWD_FIRST) {
             sfor<0, L1>([&](auto n1_) {
                 constexpr int n1 = decltype(n1_)::value;
-                v[n1] = row[n1 * RP + n2];
+                if constexpr (FH && n1 >= L1 / 4 && n1 < 3 * L1 / 4) v[n1] = make_float2(0.f, 0.f);
+                else v[n1] = row[n1 * RP + n2];
             });
         } else if constexpr (FH && KIND == PASS_FWD_MID) {
             // kept rows: element e = p + L/4 for p < L/4, p - 3L/4 for p >= 3L/4 (n_in = L/2)
