@@ -791,7 +791,11 @@ cudaError_t launch_pass(PassKind kind, const Tile& t, const LinePass& a, dim3 gr
 
 Tile pick_tile(int L, int64_t B, int64_t S, PassKind kind, bool coil_sum, int n_out, bool pair = false) {
     Tile t{};
-    if (fft2_factor(L, t.L1, t.L2, &t.list)) {
+    // One channel leaves the last inverse pass nothing adjacent to read but the line itself: the lengths of the second
+    // list from 216 points on stay with the general kernel there (432 points 12.0 us, two-phase 16.4, 576 points 12.2
+    // and 17.4; 40^2 x 108 12.3 and 14.2; from three channels on two-phase is faster, 450 points are equal).
+    const bool lone = kind == PASS_INV_LAST && S == 1 && L >= 216;
+    if (fft2_factor(L, t.L1, t.L2, &t.list) && !(lone && t.list == 1)) {
         // 8 adjacent lines (64-byte segments along the channel axis), two or three blocks per SM:
         // measured faster than 4 or 16 lines on the 640-point passes.  The coil-summing last
         // inverse pass takes 8 coils per block when its two coil chunks add into a cleared image

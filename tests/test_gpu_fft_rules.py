@@ -26,3 +26,10 @@ def _check(shape, C, maps=True, M=150):
 @pytest.mark.parametrize("shape", [(14, 256), (256, 14), (12, 512), (12, 320), (10, 8, 256)])   # staged, and 640 not
 def test_first_pass_through_shared_memory(shape, C, maps):
     _check(shape, C, maps)
+
+
+@pytest.mark.parametrize("C", [1, 2])
+@pytest.mark.parametrize("maps", [True, False])
+@pytest.mark.parametrize("shape", [(14, 100), (14, 108), (12, 288), (8, 10, 108), (108,), (216,)])   # 200 points, 216, 576
+def test_last_pass_of_a_single_channel(shape, C, maps):
+    _check(shape, C, maps)
