@@ -789,7 +789,7 @@ cudaError_t launch_pass(PassKind kind, const Tile& t, const LinePass& a, dim3 gr
                   : launch_line_pass2<0>(kind, t.L1, t.L2, a, grid, t.threads, t.smem, s);
 }
 
-Tile pick_tile(int L, int64_t B, int64_t S, PassKind kind, bool coil_sum, int n_out, bool pair = false) {
+Tile pick_tile(int D, int L, int64_t B, int64_t S, PassKind kind, bool coil_sum, int n_out, bool pair = false) {
     Tile t{};
     // One channel leaves the last inverse pass nothing adjacent to read but the line itself: the lengths of the second
     // list from 216 points on stay with the general kernel there (432 points 12.0 us, two-phase 16.4, 576 points 12.2
@@ -801,10 +801,12 @@ Tile pick_tile(int L, int64_t B, int64_t S, PassKind kind, bool coil_sum, int n_
         // inverse pass takes 8 coils per block when its two coil chunks add into a cleared image
         // (pair), else up to 16, so 16 coils need no partial-sum pass.
         int TL = (coil_sum && S > 8 && !pair) ? 16 : 8;
-        // The middle passes of lines of up to 480 points take 16: whole 128-byte lines where the elements
-        // of a line lie megabytes apart (3-D, 256 points: 607 -> 353 us forward, 238 -> 148 us inverse);
-        // with L2 = 32 only one such block would fit an SM.
-        if ((kind == PASS_FWD_MID || kind == PASS_INV_MID) && t.L2 <= 24) TL = 16;
+        // The middle passes of 3-D plans take 16 where L2 <= 24 (lengths up to 480, and 576, but not 300 and 450): whole
+        // 128-byte lines where the elements of a line lie megabytes apart (128^2 x 96, 8 coils: 482 -> 313 us forward,
+        // 479 -> 300 inverse); L2 = 25 was not measured, and with 32 only one such block would fit an SM.  In 2-D half
+        // as many blocks of twice the height cost up to 20% (160^2, 16 coils: 9.3 -> 11.0 us, 128^2, 1 coil 6.1 -> 6.8)
+        // and never gained more than 10% (288^2, 8 coils: 11.9 -> 10.8).
+        if (D == 3 && (kind == PASS_FWD_MID || kind == PASS_INV_MID) && t.L2 <= 24) TL = 16;
         t.TS = std::min<int>(TL, pow2_ceil(S));
         t.TB = std::min<int>(TL / t.TS, pow2_ceil(B));
         t.TL = t.TB * t.TS;
@@ -865,7 +867,7 @@ int forward_grids(nufft_plan_s* p, int C, int nd, int has_plain, const float2* x
         for (int e = d + 1; e < D; ++e) S *= p->K[e];
         float2* out = (d % 2 == 0) ? p->d_G : p->d_T;
         const PassKind kind = (k == 0) ? PASS_FWD_FIRST : PASS_FWD_MID;
-        Tile t = pick_tile(L, B, S, kind, false, L);
+        Tile t = pick_tile(D, L, B, S, kind, false, L);
         LinePass a{};
         a.ax = p->axis[d];
         a.n_in = (int)p->N[d];
@@ -1008,7 +1010,7 @@ int inverse_passes(nufft_plan_s* p, int C, const float2* smaps, float2* xout, cu
         const bool coil_sum = last && smaps != nullptr;
         float2* out = last ? nullptr : ((d % 2 == 0) ? tbuf : gbuf);
         const PassKind kind = last ? PASS_INV_LAST : PASS_INV_MID;
-        Tile t = pick_tile(L, B, S, kind, coil_sum, (int)p->N[d], pair);
+        Tile t = pick_tile(D, L, B, S, kind, coil_sum, (int)p->N[d], pair);
         LinePass a{};
         a.ax = p->axis[d];
         a.n_in = L;

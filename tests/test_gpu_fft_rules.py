@@ -33,3 +33,9 @@ def test_first_pass_through_shared_memory(shape, C, maps):
 @pytest.mark.parametrize("shape", [(14, 100), (14, 108), (12, 288), (8, 10, 108), (108,), (216,)])   # 200 points, 216, 576
 def test_last_pass_of_a_single_channel(shape, C, maps):
     _check(shape, C, maps)
+
+
+@pytest.mark.parametrize("C", [1, 8, 17])
+@pytest.mark.parametrize("shape", [(160, 14), (14, 10, 72), (72, 14, 10), (10, 72, 14)])   # 8 lines, 16 on each 3-D axis
+def test_middle_pass_heights(shape, C):
+    _check(shape, C)
