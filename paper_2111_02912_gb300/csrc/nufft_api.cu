@@ -815,6 +815,9 @@ Tile pick_tile(int D, int L, int64_t B, int64_t S, PassKind kind, bool coil_sum,
             t.TL *= 2;
         }
         t.threads = (t.TL * t.L2 + 31) / 32 * 32;   // ... or extra threads
+        // tiles of few lines: more threads for the image side of the first and last pass (1-D, 200 points, one coil,
+        // last inverse pass: 12.2 -> 9.1 us)
+        if (t.TL < 8) t.threads = std::max(t.threads, 160);
         // line pitch: >= L1 (L2 | 1), congruent to 16 / H mod 16 for H lines per half-warp
         const int H = std::min(t.TL, 16), want = (H == 16 ? 1 : 16 / H) % 16;
         t.LP = t.L1 * (t.L2 | 1);
