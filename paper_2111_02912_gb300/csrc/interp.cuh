@@ -226,19 +226,31 @@ __device__ __forceinline__ void gather_body(const GatherArgs& a) {
 }
 
 // Block size and resident blocks per SM that the registers are held to (0: no limit).  The gathers wait
-// on their tap loads, so warps count, as long as nothing of weight spills.  Single coils: 64-thread
-// blocks, 64 registers for one and two channel blocks (150 x 218, 5 coils, 30,011 points, VJP: 20.7 ->
-// 15.0 us).  Pairs and quads: 256 threads; the 2-D VJP and JVP pairs are held to four and three blocks
+// on their tap loads, so warps count, as long as nothing of weight spills.
+// Single coils, narrow: 64-thread blocks, 64 registers for one and two channel blocks, 80 for more, 128 for four
+// slots per lane.  Faster in 2-D (VJP 150 x 218, 5 coils, 30,011 points: 20.7 -> 15.0 us; 128^2, 9 coils, 30,000: forward
+// 15.4 -> 14.1, VJP 30.3 -> 20.4; three coils with J >= 6 and values lose: 16.6 -> 17.5) and with four slots (128^2, 33 to 128
+// coils, 20,000 points: forward 1.0 to 2.2 times as fast, JVP 1.3 to 2.5, VJP 1.15 to 1.4; 40 x 36 x 32, 96 coils: forward
+// 2.2, VJP 2.9, JVP with values 0.97).  In 3-D (40 x 36 x 32, 30,000 points) the VJP and most JVPs gain (J = 6, 9 coils: VJP
+// 178 -> 166 us, JVP 162 -> 129); the forward gains at J = 4 and 8 (9 coils: 30.7 -> 22.5, 179 -> 171) but loses
+// between (J = 7: 85.9 -> 104.5), as does the JVP with values at J = 6 (182 -> 191), and so do one to three coils at
+// J = 6 and 7 in the VJP (1 coil, J = 7: 65.8 -> 73.2) and one at J = 8 in the forward (47.4 -> 55.8).  1-D loses (200 cells,
+// 9 coils, forward: 7.7 -> 10.2 us).  All of these keep 256 threads and no limit.
+// Pairs and quads: 256 threads; the 2-D VJP and JVP pairs are held to four and three blocks
 // (VJP 40.3 -> 39.1 us on the 640^2, 16-coil case; JVP with values, 192 x 256, 12 coils, 99,999 points:
 // 69.6 -> 65.5 us).  The forward at 40 or 48 registers spills and gains nothing.
-constexpr int gather_threads(int W) { return W == 1 ? 64 : 256; }
-constexpr int gather_blocks(int D, int mode, int ND, int CPL, int W) {
-    return W == 1 ? (CPL > 1 ? 8 : ND <= 2 ? 16 : 12)
+constexpr bool gather_narrow(int D, int J, int ND, int mode, int CPL, int W) {
+    const bool fwd = mode == GM_FWD || mode == GM_FWD_SORTED;
+    return W == 1 && (CPL > 1 || D == 2 || (D == 3 && !(fwd && J >= 5 && J <= 7) && !(ND == 4 && J == 6)));
+}
+constexpr int gather_threads(bool narrow) { return narrow ? 64 : 256; }
+constexpr int gather_blocks(int D, int mode, int ND, int CPL, int W, bool narrow) {
+    return narrow ? (CPL > 1 ? 8 : ND <= 2 ? 16 : 12)
            : D == 2 && W == 2 && mode == GM_VJP ? 4
            : D == 2 && W == 2 && mode == GM_JVP ? 3 : 0;
 }
-template <int D, int J, int ND, int CPL, int MODE, int W>
-__global__ void __launch_bounds__(gather_threads(W), gather_blocks(D, MODE, ND, CPL, W)) k_gather(GatherArgs a) {
+template <int D, int J, int ND, int CPL, int MODE, int W, bool NARROW>
+__global__ void __launch_bounds__(gather_threads(NARROW), gather_blocks(D, MODE, ND, CPL, W, NARROW)) k_gather(GatherArgs a) {
     pdl_wait();
     gather_body<D, J, ND, CPL, MODE, W>(a);
 }
@@ -461,11 +473,12 @@ __global__ void __launch_bounds__(kLinesThreads, ND >= 3 ? 10 : 16) k_gather_lin
 
 template <int D, int J, int ND, int MODE>
 static cudaError_t gather_cpl(const GatherArgs& a, int cpl, cudaStream_t s) {
-    const int threads = gather_threads(cpl > 0 ? 1 : 2);
-    const int gpb = threads / a.G;
-    const unsigned blocks = (unsigned)((a.pts.m + gpb - 1) / gpb);
-    const size_t smem = (size_t)gpb * D * J * sizeof(float);
-    if (blocks == 0) return cudaSuccess;
+    if (a.pts.m == 0) return cudaSuccess;
+    constexpr bool fwd = MODE == GM_FWD || MODE == GM_FWD_SORTED;
+    auto go = [&](auto kernel, bool narrow) {
+        const int threads = gather_threads(narrow), gpb = threads / a.G;
+        (void)launch_pdl(kernel, (unsigned)((a.pts.m + gpb - 1) / gpb), threads, (size_t)gpb * D * J * sizeof(float), s, a);
+    };
     if constexpr (D > 1) {
         if (cpl == kGatherLines) {
             const int pts = kLinesThreads / 8;
@@ -475,13 +488,23 @@ static cudaError_t gather_cpl(const GatherArgs& a, int cpl, cudaStream_t s) {
         }
     }
     if (cpl == kGatherQuads) {   // coil quads (forward only)
-        if constexpr (MODE == GM_FWD || MODE == GM_FWD_SORTED) (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 4>, blocks, threads, smem, s, a);
+        if constexpr (fwd) go(k_gather<D, J, ND, 1, MODE, 4, false>, false);
         else return cudaErrorInvalidValue;
     } else if (cpl == 0) {   // coil pairs
-        (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 2>, blocks, threads, smem, s, a);
+        go(k_gather<D, J, ND, 1, MODE, 2, false>, false);
+    } else if (cpl == 1) {
+        constexpr bool narrow = gather_narrow(D, J, ND, MODE, 1, 1);
+        constexpr int few = D == 3 && narrow ? (MODE == GM_VJP && (J == 6 || J == 7) ? 3 : (fwd && J == 8 ? 1 : 0)) : 0;
+        if constexpr (few > 0) {   // up to so many coils: the other blocks
+            if (a.C <= few) {
+                go(k_gather<D, J, ND, 1, MODE, 1, false>, false);
+                return cudaGetLastError();
+            }
+        }
+        go(k_gather<D, J, ND, 1, MODE, 1, narrow>, narrow);
+    } else {
+        go(k_gather<D, J, ND, 4, MODE, 1, true>, true);   // C up to 4 G = 128
     }
-    else if (cpl == 1) (void)launch_pdl(k_gather<D, J, ND, 1, MODE, 1>, blocks, threads, smem, s, a);
-    else (void)launch_pdl(k_gather<D, J, ND, 4, MODE, 1>, blocks, threads, smem, s, a);   // C up to 4 G = 128
     return cudaGetLastError();
 }
 
