@@ -1089,9 +1089,11 @@ GatherArgs gather_args(nufft_plan_s* p, int C, int nd, int has_plain) {
     g.W = (C % 2 == 0 && C <= 64) ? 2 : 1;
     g.G = g.W == 2 ? pow2_ceil(C / 2) : std::min(32, pow2_ceil(C));
     g.lgG = ilog2(g.G);
-    // eight coils in 2-D and 3-D: whole lines (faster from one point to the largest 3-D case; its
-    // 32-bit offsets reach 4 GB of grid)
-    if (C == 8 && p->D >= 2 && p->gather_variant == NUFFT_GATHER_AUTO && p->Ktot * nd * 64 < ((int64_t)1 << 32)) g.W = 8;
+    // eight coils in 2-D and 3-D: whole lines (faster from one point to the largest 3-D case; its 32-bit offsets reach
+    // 4 GB of grid), but for the 2-D JVP with values and an odd number of taps, whose rows then end in a match of one
+    // column: 256^2, 100,000 points, J = 7 96 us, pairs 70; J = 5 51 and 42
+    const bool odd_pairs = p->D == 2 && nd == 3 && p->J % 2 == 1;
+    if (C == 8 && p->D >= 2 && !odd_pairs && p->gather_variant == NUFFT_GATHER_AUTO && p->Ktot * nd * 64 < ((int64_t)1 << 32)) g.W = 8;
     g.kb = p->kb;
     g.M = p->M;
     return g;
