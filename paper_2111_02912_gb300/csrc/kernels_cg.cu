@@ -10,7 +10,7 @@
 // kernels do; they are launch-bound up to a few hundred thousand elements.  The same algebra as
 // about twenty tensor operations per iteration kept the host busy for 340 us beside 115 us of
 // normal product (320^2, 16 coils); a solve of 10 iterations and its gradient went from 6732 to
-// 2957 us, with errors against FP64 of 6e-7 to 7e-7 (6e-7 to 1.6e-6 before).  Products and sums of the
+// 2736 us, with errors against FP64 of 6e-7 to 7e-7 (6e-7 to 1.6e-6 before).  Products and sums of the
 // scalars are FP64: the square of any FP32 number is then above zero, so <r,r> is zero only where r is,
 // and the iteration then stays where it is (alpha = beta = 0) instead of dividing zero by zero.
 #include <algorithm>
@@ -21,18 +21,25 @@ namespace nj {
 
 constexpr int kCgThreads = 256;
 
+// Sum over the block.  One warp adds 8 values a lane and then across its lanes: FP64 adds run at a low rate, and with
+// every thread shuffling five times and adding eight warp sums they took longer than the vectors (the solve and
+// gradient above: 2970 us, now 2736).
 __device__ __forceinline__ double cg_block_sum(double v) {
-    __shared__ double sh[kCgThreads / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    __syncthreads();   // sh may still be read from a previous sum
-    if (lane == 0) sh[w] = v;
+    __shared__ double sh[kCgThreads], total;
+    const int t = threadIdx.x;
+    __syncthreads();   // a previous sum may still be read
+    sh[t] = v;
     __syncthreads();
-    double t = 0.0;
+    if (t < 32) {
+        double s = sh[t];
 #pragma unroll
-    for (int k = 0; k < kCgThreads / 32; ++k) t += sh[k];
-    return t;
+        for (int k = 32; k < kCgThreads; k += 32) s += sh[t + k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (t == 0) total = s;
+    }
+    __syncthreads();
+    return total;
 }
 
 // Sum of one kernel's block partials, the same bits in every block.
