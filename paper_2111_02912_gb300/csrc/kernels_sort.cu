@@ -300,7 +300,7 @@ constexpr int kSmallBlocks = 8, kSmallThreads = 512;
 __global__ void __launch_bounds__(kSmallThreads, 1) k_sort_small(SortArgs a, int clear) {
     pdl_wait();
     __shared__ int sh[32];
-    __shared__ int s_parts[kPlanLevels], s_hmax;
+    __shared__ int s_parts[kPlanLevels], s_hmax, s_all;
     const StripTables& T = a.st;
     const int t = threadIdx.x, g = (int)blockIdx.x * kSmallThreads + t;
     constexpr int NT = kSmallBlocks * kSmallThreads;
@@ -340,7 +340,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_sort_small(SortArgs a, int
         const int lo = min(a.nunits, t * per), hi = min(a.nunits, lo + per);
         const int lgP0 = 31 - __clz(T.P);
         if (t < kPlanLevels) s_parts[t] = 0;
-        if (t == 0) s_hmax = 0;
+        if (t == 0) s_hmax = s_all = 0;
         __syncthreads();
         int hits = 0, hmax = 0, np[kPlanLevels];
 #pragma unroll
@@ -360,11 +360,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_sort_small(SortArgs a, int
             const int x = __reduce_add_sync(0xffffffffu, np[L]);
             if ((t & 31) == 0 && x) atomicAdd(&s_parts[L], x);
         }
-        const int hw = __reduce_max_sync(0xffffffffu, hmax);
-        if ((t & 31) == 0) atomicMax(&s_hmax, hw);
+        const int hw = __reduce_max_sync(0xffffffffu, hmax), ha = __reduce_add_sync(0xffffffffu, hits);
+        if ((t & 31) == 0) {
+            atomicMax(&s_hmax, hw);
+            atomicAdd(&s_all, ha);
+        }
         __syncthreads();
         int L = 0;
-        while (L < kPlanLevels - 1 && (plan_too_short(T, s_hmax, L) || s_parts[L] > T.slots)) ++L;
+        while (L < kPlanLevels - 1 && (plan_too_short(T, s_hmax, s_all, a.nunits, L) || s_parts[L] > T.slots)) ++L;
         const bool fits = s_parts[L] <= T.slots;
         const int lgP = lgP0 + L, H = fits ? s_parts[L] : 0;
         int my_parts = 0, my_whole = 0;

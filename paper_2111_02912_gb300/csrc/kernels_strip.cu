@@ -104,7 +104,7 @@ __device__ __forceinline__ void block_scan_tiles(int n, int (&carry)[V], Get get
 // --------------------------------------------------------------- sort tables
 // The plan in two launches of 256-thread blocks (unit b * 256 + t in block b, thread t).  Split
 // parts are counted for P * 2^L, L = 0..11: the smallest level whose split parts fit the partial
-// slots (and, with the default P, are long enough for the heaviest unit) is used.  (a) Per block and level: hits, split parts and whole units.  (b) Every block sums
+// slots (and, with the default P, are not too short to be worth it) is used.  (a) Per block and level: hits, split parts and whole units.  (b) Every block sums
 // the totals of the blocks before it, picks the level, scans its own units and writes their hit
 // offsets and items (split parts first: they start in the first wave), clearing the hit counts
 // (the next sort's scatter counts into them) and the fill cursors.
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_strip_plan_b(SortArgs a) {
     }
     __syncthreads();
     int L = 0;
-    while (L < kPlanLevels - 1 && (plan_too_short(T, s_tot[kPlanSums], L) || s_tot[1 + 2 * L] > T.slots)) ++L;
+    while (L < kPlanLevels - 1 && (plan_too_short(T, s_tot[kPlanSums], s_tot[0], a.nunits, L) || s_tot[1 + 2 * L] > T.slots)) ++L;
     const bool fits = s_tot[1 + 2 * L] <= T.slots;
     const int lgP = (31 - __clz(T.P)) + L;
     const int H = fits ? s_tot[1 + 2 * L] : 0;   // split parts (items of split units come first)

@@ -529,7 +529,7 @@ StripTables strip_tables(const nufft_plan_s& p) {
     t.splits = p.d_splits;
     t.nitems = p.d_nitems;
     t.P = p.strip_P;
-    t.auto_part = p.part_auto ? 1 : 0;
+    t.auto_ncg = p.part_auto ? p.ncg_max : 0;
     // by the points of this sort, not by the storage (strip_slots, never fewer): the cut into parts, and with it
     // the order of the sums, must not depend on how many points the plan has held before
     t.slots = strip_slots_for(p, std::max<int64_t>(p.M, 1));
