@@ -23,7 +23,8 @@ import torch
 
 from .plan import Plan
 
-# (spread kernel, bin shape, strip part, forward gather lanes); the tile kernel ignores the strip part
+# (spread kernel, bin shape, strip part, forward gather lanes); the tile kernel ignores the strip part, and a
+# strip part is a choice of its own: a plan's default (0) goes by the points and is not among the candidates
 CONFIG_CANDIDATES_2D = (
     ("strips", (16, 16), 64, "auto"), ("strips", (16, 16), 32, "auto"), ("strips", (16, 16), 128, "auto"),
     ("strips", (32, 32), 64, "auto"), ("tiles", (16, 16), 0, "auto"), ("tiles", (16, 32), 0, "auto"),

@@ -54,10 +54,13 @@ __device__ __forceinline__ void image_row_factors(const ImageSide& im, int64_t b
 // Registers: with L2 = 32 (256-thread blocks of 8 lines) 80 per thread, so that three blocks share
 // an SM (24 warps; the passes are issue- and latency-bound): the register DFTs fit with at most a
 // few bytes of spill (measured on the 640-point passes: FWD_MID 37.6 -> 31.5 us, INV_MID 26.4 ->
-// 22.4 us against 128 registers at two blocks per SM).  Shorter lines: 72 (L2 = 20, 24) and 64
-// (L2 <= 16); unlimited, FWD_FIRST and INV_LAST took 122-128 registers for loads in flight that a short
-// row does not have (128^2 x 96, 8 coils: FWD_FIRST 408 -> 328 us mean of the 8- and 24-channel
-// launches, INV_LAST 100 -> 68 us; 48 registers gain nothing more and cost the middle passes 6%).
+// 22.4 us against 128 registers at two blocks per SM), and 80 with L2 = 25 too.  Shorter lines: 72
+// (L2 = 20, 24) and 64 (L2 <= 18); unlimited, FWD_FIRST and INV_LAST took 122-128 registers for loads in
+// flight that a short row does not have (128^2 x 96, 8 coils: FWD_FIRST 408 -> 328 us mean of the 8- and
+// 24-channel launches, INV_LAST 100 -> 68 us; 48 registers gain nothing more and cost the middle passes 6%).
+// 72 against 128 by length: 480 points, 32 channels, middle pass 26.6 -> 22.4 us, INV_LAST 26.5 -> 20.7;
+// 400 points, INV_LAST, 32 channels 19.8 -> 18.0, but 16 channels 10.4 -> 11.0 and 480 points, one to
+// three channels 3% to 5% longer.
 // The coil-summing INV_LAST takes 8 coils per block as well when its two chunks add into the
 // image (9..16 coils: 640 blocks in 1.4 waves against 320 one-per-SM blocks of 16 coils in 2.1);
 // with more coils it runs 512-thread blocks of 16 at one block per SM.

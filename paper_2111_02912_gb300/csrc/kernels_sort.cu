@@ -291,10 +291,10 @@ __global__ void k_bin_scatter(SortArgs a) {
 
 // The whole sort of a strip plan in one launch, for few points: histogram, bin scan, scatter with the
 // hit counts, strip plan and hit lists as phases of one cluster of eight blocks, a cluster barrier
-// between two of them; the scans and the plan run in block 0.  Separate launches spend 3 to 5 us each
-// on this much work, and the host 1.5 us: 40^2,
-// 80 points: six launches of 31 us in all -> 19 us; 64^2, 4096 points: 30 -> 28 us, five launches
-// fewer.  At 30,011 points it took 107 us for 40: one point per thread is the limit.
+// between two of them; the scans and the plan (that of k_strip_plan_a and _b) run in block 0.  It saves
+// five launches at 1.5 us of host time each; on the device it takes about as long as the kernels that it
+// replaces (40^2, 80 points: 19 us, 64^2, 4096 points: 28), and the first gather waits for all of it.  At
+// 30,011 points it took 107 us for 40: one point per thread is the limit.
 constexpr int kSmallBlocks = 8, kSmallThreads = 512;
 
 __global__ void __launch_bounds__(kSmallThreads, 1) k_sort_small(SortArgs a, int clear) {

@@ -103,9 +103,10 @@ class Server:
 
     def _estimate(self, req, need_plan, batch=1):
         """Device bytes of a job: its plan (if a new one is needed) and its tensors.  A reconstruction
-        keeps y, b = E'y and the CG vectors x, r, p, F p plus one forward output per right-hand side (a
-        fused one also the coil images S x and E'E p of every right-hand side); a trajectory gradient
-        keeps y, E x, v and grad_omega."""
+        keeps y, b = E'y and the CG vectors x, r, p, F p plus one forward output per right-hand side (which
+        a strip plan's own CG passes on in the sorted order instead, within its workspace; a fused job
+        also keeps the coil images S x and E'E p of every right-hand side); a trajectory gradient keeps y,
+        E x, v and grad_omega."""
         C, M, N = int(req.smaps.shape[0]), int(req.omega.shape[1]), int(np.prod(req.shape))
         D = len(req.shape)
         if req.kind == "recon":
