@@ -462,8 +462,9 @@ __device__ __forceinline__ void gather_lines_body(const GatherArgs& a) {
 // 128^2 x 96, 8 coils, 2 M points: VJP 4570 -> 3600 us, forward 1350 -> 1230 us; 128-, 256-, 320- and
 // 640-thread blocks took 3713, 3758, 3761 and 3933 us for the VJP, 80 and 128 registers the same as 96.
 // (32-byte loads by four lanes per point ran no faster than half lines: 5130 us.)  What bounds it now
-// is the latency of the taps' L2 reads: half of them miss L1, 10 TB/s through the crossbar, at 60% of
-// the L1 pipe.
+// is the latency of the taps' L2 reads: at 64^2 x 48, 250,000 points (VJP 458 us, pairs 573) 61% of the
+// sectors miss L1, 5.9 GB come from L2 (12.9 TB/s) and the LSU data pipe runs at 62% of its peak, with
+// 9.8 cycles of long-scoreboard stalls to an issue at 19 warps per SM.
 constexpr int kLinesThreads = 64;
 template <int D, int J, int ND, int MODE>
 __global__ void __launch_bounds__(kLinesThreads, ND >= 3 ? 10 : 16) k_gather_lines(GatherArgs a) {
